@@ -250,13 +250,16 @@ void lpt_sort(std::vector<WorkItem> &it) {
 
 // Finish time of the last of `slots` resident CTAs that each take the next
 // item of the list when they are free (the work queue of the persistent
-// kernels), with item_cost as the duration.
-double queue_makespan(const std::vector<WorkItem> &it, int slots) {
+// kernels), with item_cost as the duration; with wx > 0 every item counts wx
+// columns wide (the column-owning form runs its whole tile width however few
+// columns are left at the box edge).
+double queue_makespan(const std::vector<WorkItem> &it, int slots, int wx) {
   std::priority_queue<double, std::vector<double>, std::greater<double>> q;
   for (int i = 0; i < slots; ++i) q.push(0.0);
   double m = 0.0;
   for (const WorkItem &w : it) {
-    const double t = q.top() + item_cost(w);
+    const double c = wx > 0 ? double(wx) * (w.ny + 2) * (w.nz + 3) : item_cost(w);
+    const double t = q.top() + c;
     q.pop();
     q.push(t);
     m = std::max(m, t);
@@ -266,6 +269,14 @@ double queue_makespan(const std::vector<WorkItem> &it, int slots) {
 
 constexpr int kWhole = 1 << 30;
 constexpr int kRestChunk = 16;  // planes of the chunks a long column's rest is cut into
+// Short even chunks, tried where a level has at most kShortTiles tile per
+// CTA (a level with more fills the machine with whole columns, and the extra
+// plane steps of short chunks only cost it).  Measured per advance, chunks of
+// at least 16 planes against these: one 32^3 box, mixed, 16 x 8 tiles
+// 167 -> 50 us (128 CTAs busy instead of 16); the FP64 Sod tube 128 x 8 x 8
+// 4.95 -> 1.16 ms (64 busy instead of 8); a 32^3 box, FP64, 19.2 -> 2.4 ms.
+constexpr int kShortChunks[] = {14, 12, 10, 8, 6, 5, 4, 3, 2, 1};
+constexpr size_t kShortTiles = 1, kShortItems = 8;
 
 // Every box cut into tx x ty column tiles, every column of n planes cut by
 // the rule (L, M): n > M gives a main chunk of M planes and the rest in
@@ -311,14 +322,16 @@ std::vector<WorkItem> tile_items(const std::vector<std::array<int, 3>> &n, int t
 // column (a chunk starts with its own ring prologue), so when whole columns leave
 // the `slots` resident CTAs unevenly loaded (fewer tiles than CTAs, or a
 // last partial wave), the columns are cut along z: among even cuts into
-// chunks of at least 16 planes and cuts into one main chunk plus short
-// rest chunks that fill the queue's tail, the one with the earliest
-// simulated finish is taken, if it beats whole columns by 2 %.
+// chunks of at least 16 planes, on small levels even cuts down to one plane,
+// and cuts into one main chunk plus short rest chunks that fill the queue's
+// tail, the one with the earliest simulated finish is taken, if it beats
+// whole columns by 2 %.
 std::vector<WorkItem> task_items(const std::vector<std::array<int, 3>> &n, int tx, int ty,
-                                 int slots, bool chunk) {
+                                 int slots, bool chunk, bool full_width = false) {
   std::vector<WorkItem> best = tile_items(n, tx, ty, kWhole, kWhole);
   if (!chunk || slots < 1 || best.empty()) return best;
-  const double whole = queue_makespan(best, slots);
+  const int wx = full_width ? tx + 2 : 0;
+  const double whole = queue_makespan(best, slots, wx);
   double total = 0.0;
   for (const WorkItem &w : best) total += item_cost(w);
   if (whole <= 1.02 * total / slots) return best;
@@ -337,24 +350,83 @@ std::vector<WorkItem> task_items(const std::vector<std::array<int, 3>> &n, int t
   std::sort(rules.begin(), rules.end());
   rules.erase(std::unique(rules.begin(), rules.end()), rules.end());
 
-  const size_t cap = (size_t)64 * slots;
+  const size_t cap = (size_t)64 * slots, tiles = best.size();
   double bm = 0.98 * whole;
   for (const auto &r : rules) {
     std::vector<WorkItem> it = tile_items(n, tx, ty, r.first, r.second);
     if (it.size() > std::max(cap, best.size())) continue;
-    const double m = queue_makespan(it, slots);
+    const double m = queue_makespan(it, slots, wx);
     if (m < bm) {
       bm = m;
       best.swap(it);
     }
   }
+  if (tiles <= (size_t)kShortTiles * slots)
+    for (int L : kShortChunks) {  // from long to short: each has to gain 2 % on the one before
+      if (L >= nmax) continue;
+      std::vector<WorkItem> it = tile_items(n, tx, ty, L, kWhole);
+      if (it.size() > (size_t)kShortItems * slots) break;
+      const double m = queue_makespan(it, slots, wx);
+      if (m < 0.98 * bm) {
+        bm = m;
+        best.swap(it);
+      }
+    }
   return best;
 }
 
-std::vector<WorkItem> build_items(const nyx_plan &P, int tx, int ty, int slots, bool chunk) {
-  std::vector<std::array<int, 3>> n(P.nbox);
-  for (int b = 0; b < P.nbox; ++b) n[b] = {P.hbox[b].n[0], P.hbox[b].n[1], P.hbox[b].n[2]};
-  return task_items(n, tx, ty, slots, chunk);
+// Items regrouped by the box groups [gb[g], gb[g+1]), each group in list
+// order; off gets the first item of each group after the 0 it starts with.
+void group_items(const std::vector<WorkItem> &items, const std::vector<int> &gb,
+                 std::vector<WorkItem> &out, std::vector<int> &off) {
+  out.reserve(items.size());
+  for (size_t g = 0; g + 1 < gb.size(); ++g) {
+    for (const WorkItem &w : items)
+      if (w.box >= gb[g] && w.box < gb[g + 1]) out.push_back(w);
+    off.push_back((int)out.size());
+  }
+}
+
+// The work list of one tile shape, made when the shape is first chosen (plan
+// creation, nyx_hydro_set_tile_shape, the autotuner): a plan runs one shape,
+// and simulating the queues of all of them took most of a plan's set-up.
+// Relaxed capture mode: the allocation and the upload touch no stream that a
+// caller may be capturing.
+int ensure_items(nyx_plan *P, int s) {
+  if (P->d_items[s]) return NYX_OK;
+  std::vector<std::array<int, 3>> n(P->nbox);
+  for (int b = 0; b < P->nbox; ++b) n[b] = {P->hbox[b].n[0], P->hbox[b].n[1], P->hbox[b].n[2]};
+  const TileShape ts = fused_shape(s);
+  std::vector<WorkItem> it =
+      task_items(n, ts.tx, ts.ty, P->max_grid[s], P->prm.z_chunks != 0, !ts.task);
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  CK(cudaThreadExchangeStreamCaptureMode(&mode));
+  auto upload = [&](const std::vector<WorkItem> &v, WorkItem **d) {
+    cudaError_t e = cudaMalloc(d, sizeof(WorkItem) * std::max<size_t>(1, v.size()));
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpy(*d, v.data(), sizeof(WorkItem) * v.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      cudaFree(*d);
+      *d = nullptr;
+    }
+    return e;
+  };
+  cudaError_t e = cudaSuccess;
+  if (P->ngrp > 1) {  // box groups are set up already: this shape's items by group
+    std::vector<WorkItem> by;
+    std::vector<int> off(1, 0);
+    group_items(it, P->grp_box, by, off);
+    e = upload(by, &P->d_items_grp[s]);
+    if (e == cudaSuccess) P->grp_off[s] = off;
+  }
+  if (e == cudaSuccess) e = upload(it, &P->d_items[s]);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess)
+    return e == cudaErrorMemoryAllocation ? fail(NYX_ENOMEM, "work list allocation failed")
+                                          : cuda_fail(e, "work list upload");
+  P->nitems[s] = (int)it.size();
+  P->h_items[s] = std::move(it);
+  return NYX_OK;
 }
 
 void free_plan(nyx_plan *P) {
@@ -702,15 +774,9 @@ int do_advance(nyx_plan *P, nyx_level *L, const double *a_old, const double *a_n
 
 // A part's items regrouped by the read-back groups [gb[g], gb[g+1]) of boxes.
 int part_groups(nyx_plan::RunPart &pt, const std::vector<int> &gb) {
-  const int ng = (int)gb.size() - 1;
   std::vector<WorkItem> it;
-  it.reserve(pt.h_items.size());
   pt.grp_off.assign(1, 0);
-  for (int g = 0; g < ng; ++g) {
-    for (const WorkItem &w : pt.h_items)
-      if (w.box >= gb[g] && w.box < gb[g + 1]) it.push_back(w);
-    pt.grp_off.push_back((int)it.size());
-  }
+  group_items(pt.h_items, gb, it, pt.grp_off);
   cudaFree(pt.d_items_grp);
   pt.d_items_grp = nullptr;
   CK(cudaMalloc(&pt.d_items_grp, sizeof(WorkItem) * std::max<size_t>(1, it.size())));
@@ -722,17 +788,22 @@ int part_groups(nyx_plan::RunPart &pt, const std::vector<int> &gb) {
 // advance and read-back overlapped per group) and by nyx_hydro_run (each
 // group's ghost fill beside the other groups' advances): up to 32 ranges of
 // whole boxes with about equal cells (the groups' bit masks are 32 bits), as
-// long as each group keeps 2 waves of items or more in the plan's tile shape.
-// One group (no overlap) otherwise.  Every shape gets the same groups.  (On the 512^3 large level: 32 groups 1.74e9 zone-updates/s end
-// to end, 16 groups 1.72e9, 8 groups 1.59e9.)
-int setup_readback(nyx_plan *P) {
+// long as each group keeps 2 waves of items or more in the plan's tile shape
+// (4 waves of the task form's half-size items for a run on the device, where a
+// group's tail costs more than its overlapped fill gains: 563 boxes, two
+// steps, 32.0 ms with 9 groups, 32.1 ms with 18).  One group (no overlap)
+// otherwise.  Every shape gets the same groups.  (On the 512^3 large level:
+// 32 groups 1.74e9 zone-updates/s end to end, 16 groups 1.72e9, 8 groups
+// 1.59e9.)
+int setup_readback(nyx_plan *P, bool host) {
   const int nsh = fused_num_shapes(P->prm.precision);
   int waves = P->nitems[P->shape] / std::max(1, P->max_grid[P->shape]);
   if (!P->parts.empty()) {
     waves = 0;
     for (const auto &pt : P->parts) waves += pt.nitems / std::max(1, pt.grid);
   }
-  const int G = std::min(std::min(32, P->nbox), waves / 2);
+  const int per = host ? 2 : (fused_shape(P->shape).task ? 4 : 2);
+  const int G = std::min(std::min(32, P->nbox), waves / per);
   std::vector<int> gb(1, 0);
   for (int g = 1; g < G; ++g) {
     const long long want = P->total_cells * g / G;
@@ -749,14 +820,10 @@ int setup_readback(nyx_plan *P) {
   P->ngrp = 1;
   if (ng < 2) return NYX_OK;
   for (int s = 0; s < nsh; ++s) {
+    if (!P->d_items[s]) continue;  // not chosen yet: grouped when it is
     std::vector<WorkItem> it;
-    it.reserve(P->h_items[s].size());
     P->grp_off[s].assign(1, 0);
-    for (int g = 0; g < ng; ++g) {
-      for (const WorkItem &w : P->h_items[s])
-        if (w.box >= gb[g] && w.box < gb[g + 1]) it.push_back(w);
-      P->grp_off[s].push_back((int)it.size());
-    }
+    group_items(P->h_items[s], gb, it, P->grp_off[s]);
     CK(cudaMalloc(&P->d_items_grp[s], sizeof(WorkItem) * it.size()));
     CK(cudaMemcpy(P->d_items_grp[s], it.data(), sizeof(WorkItem) * it.size(),
                   cudaMemcpyHostToDevice));
@@ -1016,13 +1083,13 @@ void tune_cache_save(const std::string &path, const std::map<std::string, TuneCh
 // Items of the boxes `sel` (indices into the plan's box list) for one tile
 // shape, with the box indices of the plan.
 std::vector<WorkItem> subset_items(const nyx_plan &P, const std::vector<int> &sel, int tx, int ty,
-                                   int slots, bool chunk) {
+                                   int slots, bool chunk, bool full_width = false) {
   std::vector<std::array<int, 3>> n(sel.size());
   for (size_t k = 0; k < sel.size(); ++k) {
     const BoxDev &X = P.hbox[sel[k]];
     n[k] = {X.n[0], X.n[1], X.n[2]};
   }
-  std::vector<WorkItem> it = task_items(n, tx, ty, slots, chunk);
+  std::vector<WorkItem> it = task_items(n, tx, ty, slots, chunk, full_width);
   for (WorkItem &w : it) w.box = sel[w.box];
   return it;
 }
@@ -1157,14 +1224,15 @@ int tune_shape(nyx_plan *P, const FusedArgs &base) {
   for (auto it = gcells.begin(); it != gcells.end(); ++it)
     if (it->second > biggest->second) biggest = it;
   P->shape = biggest->first.first;
-  if (groups.size() == 1 && biggest->first.second * nsm >= P->max_grid[P->shape]) return NYX_OK;
+  if (groups.size() == 1 && biggest->first.second * nsm >= P->max_grid[P->shape])
+    return ensure_items(P, P->shape);
   for (auto &kv : groups) {
     nyx_plan::RunPart pt;
     pt.shape = kv.first.first;
     pt.grid = std::min(P->max_grid[pt.shape], kv.first.second * nsm);
     std::sort(kv.second.begin(), kv.second.end());
     const TileShape ts = fused_shape(pt.shape);
-    pt.h_items = subset_items(*P, kv.second, ts.tx, ts.ty, pt.grid, P->prm.z_chunks != 0);
+    pt.h_items = subset_items(*P, kv.second, ts.tx, ts.ty, pt.grid, P->prm.z_chunks != 0, !ts.task);
     pt.nitems = (int)pt.h_items.size();
     CK(cudaMalloc(&pt.d_items, sizeof(WorkItem) * std::max(1, pt.nitems)));
     CK(cudaMemcpy(pt.d_items, pt.h_items.data(), sizeof(WorkItem) * pt.nitems,
@@ -1564,15 +1632,14 @@ int nyx_hydro_plan(const nyx_level_desc *lev, const nyx_hydro_params *prm, void 
           goto fail_out;
         }
       }
-      for (int s = 0; s < fused_num_shapes(prm->precision); ++s) {
-        TileShape ts = fused_shape(s);
-        std::vector<WorkItem> it = build_items(*P, ts.tx, ts.ty, P->max_grid[s], prm->z_chunks);
-        P->nitems[s] = (int)it.size();
-        TRYC(cudaMalloc(&P->d_items[s], sizeof(WorkItem) * it.size()));
-        TRYC(cudaMemcpy(P->d_items[s], it.data(), sizeof(WorkItem) * it.size(),
-                        cudaMemcpyHostToDevice));
-        P->h_items[s] = std::move(it);
-      }
+      // An untuned mixed plan starts with the 16 x 8 task form: per advance it
+      // beat the 16 x 16 column-owning form at every size measured (us, column
+      // form / task form: 16^3 83 / 40, 32^3 85 / 50, 64^3 332 / 169, 128^3
+      // 2161 / 1050, 8 boxes of 50^3 2005 / 736, 216 boxes of 32^3 7334 / 3662)
+      // and the other task shapes at all but the smallest, where they tie.
+      // FP64 has only the column-owning form, whose shapes lie within 10 %.
+      P->shape = prm->precision == NYX_MIXED ? 3 : 0;
+      TRY(ensure_items(P, P->shape));
       TRYC(cudaMalloc(&P->d_queue, sizeof(int)));
       TRYC(cudaMemset(P->d_queue, 0, sizeof(int)));
       TRYC(cudaGetLastError());
@@ -1661,14 +1728,14 @@ int nyx_hydro_run(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev
   // box groups (made once, outside any capture): a run overlaps each group's
   // ghost fill with the other groups' advances
   if (P->prm.batching != NYX_PER_BOX && P->ngrp == 0)
-    if (int rc = setup_readback(P)) return rc;
+    if (int rc = setup_readback(P, false)) return rc;
   if (!use_graph) return enqueue_run(P, L, a_dev, dt_dev, nsteps, compute_dt0);
   if (P->prm.batching == NYX_PERSISTENT && P->prm.autotune && !P->tuned) {
     // tune outside the capture: one eager step on scratch copies is not
     // possible without the caller's buffers, so tune on the real ones and
     // redo the work below (the tuning launches only write state[1-cur]).
     FusedArgs a{};
-    a.boxes = P->d_boxes;
+      a.boxes = P->d_boxes;
     a.queue = P->d_queue;
     a.K = P->d_K;
     a.SC = P->d_SC;
@@ -1781,7 +1848,7 @@ int nyx_hydro_step_host_valid(nyx_plan *P, nyx_level *L, const double *host_in, 
     P->plane_pref = pp;
   }
   if (P->prm.batching != NYX_PER_BOX && P->ngrp == 0)
-    if (int rc = setup_readback(P)) return rc;
+    if (int rc = setup_readback(P, true)) return rc;
   if (P->prm.batching != NYX_PER_BOX && !(P->prm.autotune && !P->tuned)) prepare_tmaps(P, L);
   const size_t bytes = sizeof(double) * NCONS * (size_t)P->total_cells;
   double h[3] = {a_old, a_new, *dt_inout};
@@ -1865,6 +1932,7 @@ int nyx_hydro_set_tile_shape(nyx_plan *P, int shape) {
   if (!P) return fail(NYX_EINVAL, "null plan");
   if (P->prm.batching != NYX_PERSISTENT) return fail(NYX_EINVAL, "plan is not persistent");
   if (shape < 0 || shape >= fused_num_shapes(P->prm.precision)) return fail(NYX_EINVAL, "tile shape out of range");
+  if (int rc = ensure_items(P, shape)) return rc;
   for (auto &pt : P->parts) {
     cudaFree(pt.d_items);
     cudaFree(pt.d_items_grp);
