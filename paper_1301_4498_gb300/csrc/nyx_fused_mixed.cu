@@ -81,19 +81,17 @@ __global__ void k_estdt_mixed(const BoxDev *boxes, const long long *cell_pref, i
   const float small_pres = nyx_mixed::d2f_rn(K->small_pres);
   const double a = *a_dev;
   float local_min = __int_as_float(0x7f800000);
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    int lo = 0, hi = nbox - 1;
-    while (lo < hi) {
-      int mid = (lo + hi + 1) >> 1;
-      if (cell_pref[mid] <= t) lo = mid; else hi = mid - 1;
+  int box = -1;
+  float adx[3] = {0.0f, 0.0f, 0.0f};  // a dx of the current box (FP64 products)
+  for (CellWalk w(cell_pref, nbox, total); w.valid(); w.next(cell_pref, nbox)) {
+    const BoxDev &b = boxes[w.box];
+    if (w.box != box) {
+      box = w.box;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) adx[d] = (float)(a * b.dx[d]);
     }
-    const BoxDev b = boxes[lo];
-    const long long f = t - cell_pref[lo];
-    const int i = (int)(f % b.n[0]);
-    const long long u = f / b.n[0];
-    const int j = (int)(u % b.n[1]);
-    const int kk = (int)(u / b.n[1]);
+    int i, j, kk;
+    w.cell(cell_pref, b, i, j, kk);
     const double *S = state + NCONS * b.pref;
     const long long id = cell_index(b, i, j, kk);
     const float rho = nyx_mixed::d2f_rn(S[id]);
@@ -104,8 +102,7 @@ __global__ void k_estdt_mixed(const BoxDev *boxes, const long long *cell_pref, i
     const float c = c2 * rsqrtf(c2);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const float adx = nyx_mixed::d2f_rn(a * b.dx[d]);
-      const float tt = adx / (fabsf(nyx_mixed::d2f_rn(S[(1 + d) * b.stride + id]) * ir) + c);
+      const float tt = adx[d] / (fabsf(nyx_mixed::d2f_rn(S[(1 + d) * b.stride + id]) * ir) + c);
       local_min = fminf(local_min, tt);
     }
   }
@@ -119,10 +116,8 @@ __global__ void k_estdt_mixed(const BoxDev *boxes, const long long *cell_pref, i
 void launch_estdt_mixed(const BoxDev *boxes, const long long *cell_pref, int nbox, long long total,
                         const double *state, const SchemeConsts *K, const double *a_dev,
                         unsigned long long *dtacc, cudaStream_t st) {
-  long long g = (total + 255) / 256;
-  if (g > 152 * 64) g = 152 * 64;
-  if (g < 1) g = 1;
-  k_estdt_mixed<<<(int)g, 256, 0, st>>>(boxes, cell_pref, nbox, total, state, K, a_dev, dtacc);
+  k_estdt_mixed<<<walk_grid(total, 256), 256, 0, st>>>(boxes, cell_pref, nbox, total, state, K,
+                                                       a_dev, dtacc);
 }
 
 }  // namespace nyx

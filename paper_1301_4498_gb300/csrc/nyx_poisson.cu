@@ -59,31 +59,13 @@ __device__ __forceinline__ T resid_at(const T *phi, const T *f, const Dims &d, T
   return f[id] - (nbsum(phi, d, i, j, k) - T(6) * phi[id]) * ih2;
 }
 
-// valid cell t of the level (box by binary search of the cell offsets)
-__device__ __forceinline__ void level_cell(const BoxDev *boxes, const long long *cell_pref,
-                                           int nbox, long long t, int &b, int &i, int &j,
-                                           int &k) {
-  int lo = 0, hi = nbox - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (cell_pref[mid] <= t) lo = mid; else hi = mid - 1;
-  }
-  b = lo;
-  const BoxDev &X = boxes[lo];
-  const long long f = t - cell_pref[lo];
-  i = (int)(f % X.n[0]);
-  const long long u = f / X.n[0];
-  j = (int)(u % X.n[1]);
-  k = (int)(u / X.n[1]);
-}
-
 __global__ void k_pg_gather(const double *state, const BoxDev *boxes, const long long *cell_pref,
                             const int *box_lo, int nbox, long long total, Dims d, double *f) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    int b, i, j, k;
-    level_cell(boxes, cell_pref, nbox, t, b, i, j, k);
-    const BoxDev X = boxes[b];
+  for (CellWalk w(cell_pref, nbox, total); w.valid(); w.next(cell_pref, nbox)) {
+    const int b = w.box;
+    const BoxDev &X = boxes[b];
+    int i, j, k;
+    w.cell(cell_pref, X, i, j, k);
     f[didx(d, box_lo[3 * b] + i, box_lo[3 * b + 1] + j, box_lo[3 * b + 2] + k)] =
         state[NCONS * X.pref + cell_index(X, i, j, k)];
   }
@@ -220,8 +202,8 @@ __global__ void k_pm_kick(const double *x, double *u, long long np, const double
     gm = fmax(gm, __shfl_xor_sync(0xffffffffu, gm, o));
   }
   if ((threadIdx.x & 31) == 0) {
-    atomicMax(&mx[0], (unsigned long long)__double_as_longlong(um));
-    atomicMax(&mx[1], (unsigned long long)__double_as_longlong(gm));
+    atomic_max_pos(&mx[0], um);
+    atomic_max_pos(&mx[1], gm);
   }
 }
 
@@ -244,8 +226,8 @@ __global__ void k_pm_maxes(const double *x, const double *u, long long np, const
     gm = fmax(gm, __shfl_xor_sync(0xffffffffu, gm, o));
   }
   if ((threadIdx.x & 31) == 0) {
-    atomicMax(&mx[0], (unsigned long long)__double_as_longlong(um));
-    atomicMax(&mx[1], (unsigned long long)__double_as_longlong(gm));
+    atomic_max_pos(&mx[0], um);
+    atomic_max_pos(&mx[1], gm);
   }
 }
 
@@ -296,8 +278,7 @@ __global__ void k_pg_rhs(double *f, long long n, const double *mean, double c,
     loc = fmax(loc, fabs(v));
   }
   for (int o = 16; o > 0; o >>= 1) loc = fmax(loc, __shfl_xor_sync(0xffffffffu, loc, o));
-  if ((threadIdx.x & 31) == 0)
-    atomicMax(fmax_bits, (unsigned long long)__double_as_longlong(loc));
+  if ((threadIdx.x & 31) == 0) atomic_max_pos(fmax_bits, loc);
 }
 
 // one colour of a red-black sweep: cells with (i + j + k) % 2 == color
@@ -319,7 +300,7 @@ __global__ void k_pg_resid_max(const double *phi, const double *f, Dims d, doubl
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < d.n[0]) loc = fabs(resid_at(phi, f, d, ih2, i, (int)blockIdx.y, (int)blockIdx.z));
   for (int o = 16; o > 0; o >>= 1) loc = fmax(loc, __shfl_xor_sync(0xffffffffu, loc, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(loc));
+  if ((threadIdx.x & 31) == 0) atomic_max_pos(out, loc);
 }
 
 // coarse f = mean of the 8 fine residuals (index order), coarse phi = 0
@@ -385,8 +366,7 @@ __global__ void k_pg_resid32(const double *phi, const double *f, Dims d, double 
     loc = fabsf(v32);
   }
   for (int o = 16; o > 0; o >>= 1) loc = fmaxf(loc, __shfl_xor_sync(0xffffffffu, loc, o));
-  if ((threadIdx.x & 31) == 0)
-    atomicMax(out, (unsigned long long)__double_as_longlong((double)loc));
+  if ((threadIdx.x & 31) == 0) atomic_max_pos(out, (double)loc);
 }
 
 // phi += e (the FP32 correction), in FP64
@@ -679,11 +659,11 @@ __global__ void __launch_bounds__(kSwThreads) k_pg_smooth(const float *phi_in, c
 __global__ void k_pg_grav(const double *u, Dims d, double hdx, const BoxDev *boxes,
                           const long long *cell_pref, const int *box_lo, int nbox,
                           long long total, double *grav) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    int b, i, j, k;
-    level_cell(boxes, cell_pref, nbox, t, b, i, j, k);
-    const BoxDev X = boxes[b];
+  for (CellWalk w(cell_pref, nbox, total); w.valid(); w.next(cell_pref, nbox)) {
+    const int b = w.box;
+    const BoxDev &X = boxes[b];
+    int i, j, k;
+    w.cell(cell_pref, X, i, j, k);
     const int I = box_lo[3 * b] + i, J = box_lo[3 * b + 1] + j, K = box_lo[3 * b + 2] + k;
     double *G = grav + NGRAV * X.pref + cell_index(X, i, j, k);
     G[0] = -((u[didx(d, wrp(I + 1, d.n[0]), J, K)] - u[didx(d, wrp(I - 1, d.n[0]), J, K)]) * hdx);
@@ -1096,9 +1076,9 @@ int nyx_poisson_solve(nyx_poisson *S, const double *state, const double *rho_dm,
   const long long N = (long long)g0.d.n[0] * g0.d.n[1] * g0.d.n[2];
   cudaStream_t st = P.stream;
   if (!warm_start) CK(cudaMemsetAsync(g0.phi, 0, N * sizeof(double), st));
-  k_pg_gather<<<gridn(P.total_cells, 256), 256, 0, st>>>(state, P.d_boxes, P.d_cell_pref,
-                                                        S->d_box_lo, P.nbox, P.total_cells, g0.d,
-                                                        g0.f);
+  k_pg_gather<<<walk_grid(P.total_cells, 256), 256, 0, st>>>(state, P.d_boxes, P.d_cell_pref,
+                                                            S->d_box_lo, P.nbox, P.total_cells,
+                                                            g0.d, g0.f);
   if (rho_dm) {
     k_pg_add<<<gridn(N, 256), 256, 0, st>>>(g0.f, rho_dm, N);
     S->launches += 1;
@@ -1122,7 +1102,7 @@ int nyx_poisson_solve(nyx_poisson *S, const double *state, const double *rho_dm,
     if ((rc = resid_max(S, &res))) return rc;
   }
   if (grav_out) {
-    k_pg_grav<<<gridn(P.total_cells, 256), 256, 0, st>>>(g0.phi, g0.d, 0.5 / S->dx, P.d_boxes,
+    k_pg_grav<<<walk_grid(P.total_cells, 256), 256, 0, st>>>(g0.phi, g0.d, 0.5 / S->dx, P.d_boxes,
                                                         P.d_cell_pref, S->d_box_lo, P.nbox,
                                                         P.total_cells, grav_out);
     S->launches += 1;

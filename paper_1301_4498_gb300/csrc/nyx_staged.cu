@@ -318,19 +318,10 @@ __global__ void k_correct(const BoxDev *boxes, const long long *cell_pref, int n
   const StepConsts sc = *SC;
   double local_min = __longlong_as_double(0x7ff0000000000000LL);
   unsigned flags = 0;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    int lo = 0, hi = nbox - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (cell_pref[mid] <= t) lo = mid; else hi = mid - 1;
-    }
-    const BoxDev b = boxes[lo];
-    const long long f = t - cell_pref[lo];
-    const int i = (int)(f % b.n[0]);
-    const long long u = f / b.n[0];
-    const int j = (int)(u % b.n[1]);
-    const int kk = (int)(u / b.n[1]);
+  for (CellWalk w(cell_pref, nbox, total); w.valid(); w.next(cell_pref, nbox)) {
+    const BoxDev &b = boxes[w.box];
+    int i, j, kk;
+    w.cell(cell_pref, b, i, j, kk);
     const long long bs = b.stride;
     const long long id = NCONS * b.pref + cell_index(b, i, j, kk);
     const long long ig = NGRAV * b.pref + cell_index(b, i, j, kk);
@@ -416,19 +407,10 @@ __global__ void k_estdt(const BoxDev *boxes, const long long *cell_pref, int nbo
   const SchemeConsts k = *K;
   const double a = *a_dev;
   double local_min = __longlong_as_double(0x7ff0000000000000LL);
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    int lo = 0, hi = nbox - 1;
-    while (lo < hi) {
-      int mid = (lo + hi + 1) >> 1;
-      if (cell_pref[mid] <= t) lo = mid; else hi = mid - 1;
-    }
-    const BoxDev b = boxes[lo];
-    long long f = t - cell_pref[lo];
-    int i = (int)(f % b.n[0]);
-    long long u = f / b.n[0];
-    int j = (int)(u % b.n[1]);
-    int kk = (int)(u / b.n[1]);
+  for (CellWalk w(cell_pref, nbox, total); w.valid(); w.next(cell_pref, nbox)) {
+    const BoxDev &b = boxes[w.box];
+    int i, j, kk;
+    w.cell(cell_pref, b, i, j, kk);
     const double *S = state + NCONS * b.pref;
     long long id = cell_index(b, i, j, kk);
     const double rho = S[id];
@@ -513,7 +495,7 @@ void launch_step_setup(const SchemeConsts *K, const double *a_old, const double 
 void launch_estdt(const BoxDev *boxes, const long long *cell_pref, int nbox, long long total,
                   const double *state, const SchemeConsts *K, const double *a_dev,
                   unsigned long long *dtacc, cudaStream_t st) {
-  k_estdt<<<grid_for(total, 256), 256, 0, st>>>(boxes, cell_pref, nbox, total, state, K, a_dev,
+  k_estdt<<<walk_grid(total, 256), 256, 0, st>>>(boxes, cell_pref, nbox, total, state, K, a_dev,
                                                  dtacc);
 }
 
@@ -523,10 +505,10 @@ void launch_correct(const BoxDev *boxes, const long long *cell_pref, int nbox, l
                     unsigned *status, bool f32_dt, cudaStream_t st) {
   if (total <= 0) return;
   if (f32_dt)
-    k_correct<true><<<grid_for(total, 256), 256, 0, st>>>(boxes, cell_pref, nbox, total, K, SC, S,
+    k_correct<true><<<walk_grid(total, 256), 256, 0, st>>>(boxes, cell_pref, nbox, total, K, SC, S,
                                                            Sp, Go, Gn, dtacc, status);
   else
-    k_correct<false><<<grid_for(total, 256), 256, 0, st>>>(boxes, cell_pref, nbox, total, K, SC, S,
+    k_correct<false><<<walk_grid(total, 256), 256, 0, st>>>(boxes, cell_pref, nbox, total, K, SC, S,
                                                             Sp, Go, Gn, dtacc, status);
 }
 
