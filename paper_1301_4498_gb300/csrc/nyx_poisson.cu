@@ -12,12 +12,14 @@
 // domain; the 8 children in index order) and the residual norm is a max,
 // so the result does not depend on scheduling.  FP64 throughout by default;
 // this unit is built without FMA contraction.  Mixed precision (on request):
-// iterative refinement, each cycle an FP64 residual r = f - L phi, one FP32
-// V-cycle of the same multigrid on L e = r from e = 0, and phi += e in FP64;
-// the stopping test is the max norm of that residual (rounded to float).
+// iterative refinement, each cycle a residual r = f - L phi, one FP32 V-cycle
+// of the same multigrid on L e = r from e = 0, and phi += e, with phi and r's
+// sums in 64-bit fixed point (or in FP64 where no scale fits); the stopping
+// test is the max norm of that residual (rounded to float).
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -376,6 +378,147 @@ __global__ void k_pg_correct(double *phi, const float *e, long long n) {
     phi[t] = phi[t] + (double)e[t];
 }
 
+// ---------------------------------------------------------------- fixed point
+// The refinement solve's potential and right-hand side as 64-bit integers: phi
+// in units of 1/s, s a power of two that puts a bound of every potential the
+// solve can meet near 2^62, and h^2 f in units of 1/(s 2^K), K what its own
+// maximum leaves (it is smaller than the potential by up to n^2).  The
+// residual's seven terms then add exactly (modulo 2^64) on the integer pipe,
+// and phi += e loses nothing but e's own last bits, while in FP64 the
+// residual's 7 operations a cell alone take this part's FP64 pipe 187 us on a
+// 256^3 grid and round at 2^-53 of the potential.
+
+// float -> fixed, nearest: |e s| as hi 2^32 + lo, both exact in FP32 (a
+// negative number's low half, 2^32 - x, would not be)
+__device__ __forceinline__ long long to_fix(float e, float s) {
+  const float v = fabsf(e) * s;
+  const float h = floorf(v * 2.3283064365386963e-10f);  // 2^-32
+  const unsigned lo = __float2uint_rn(fmaf(-h, 4294967296.0f, v));
+  const long long m = ((long long)__float2int_rz(h) << 32) + lo;
+  return e < 0.0f ? -m : m;
+}
+// fixed -> float (sign and magnitude: no cancellation between the halves)
+__device__ __forceinline__ float from_fix(long long v) {
+  const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
+  const float f = fmaf((float)(unsigned)(m >> 32), 4294967296.0f, (float)(unsigned)m);
+  return v < 0 ? -f : f;
+}
+
+// The right-hand side in fixed point (scale s, in place) and, from phi = 0, the
+// first residual: f itself (r null from a given phi)
+__global__ void k_pg_rhs_fix(const double *f, long long *ff, long long n, double s, long long *phi,
+                             float *r) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
+       t += (long long)gridDim.x * blockDim.x) {
+    const double v = f[t];
+    ff[t] = __double2ll_rn(v * s);
+    if (r) {
+      phi[t] = 0;
+      r[t] = (float)v;
+    }
+  }
+}
+__global__ void k_pg_to_fix(const double *x, long long *y, long long n, double s) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
+       t += (long long)gridDim.x * blockDim.x)
+    y[t] = __double2ll_rn(x[t] * s);
+}
+__global__ void k_pg_from_fix(const long long *y, double *x, long long n, double is) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
+       t += (long long)gridDim.x * blockDim.x)
+    x[t] = (double)y[t] * is;
+}
+__global__ void k_pg_absmax(const double *x, long long n, unsigned long long *out) {
+  unsigned long long loc = 0;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
+       t += (long long)gridDim.x * blockDim.x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x[t]) & ~(1ull << 63);
+    loc = loc > b ? loc : b;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long b = __shfl_xor_sync(0xffffffffu, loc, o);
+    loc = loc > b ? loc : b;
+  }
+  if ((threadIdx.x & 31) == 0) atomic_max_pos(out, __longlong_as_double((long long)loc));
+}
+
+// Residual r = f - L phi of the finest grid as float, and the max norm of it.
+// h^2 r = f 2^-K + 6 phi - (neighbours) keeps f's K extra bits where the sum of
+// the others leaves room for them (|.| < 2^(62-K)), else they are below its
+// rounding to float; c = 1 / (h^2 s).
+//
+// Bound: memory.  A thread marches zc planes with the cells above and below in
+// registers, two cells of a row at a time where rows are even (PAIR): 19 B a
+// cell from L2.  One thread per cell read 59 B a cell: 164 us on a 256^3 grid
+// (324 MB of DRAM), 86 us this way.
+constexpr int kRfX = 32, kRfY = 8;
+template <bool PAIR>
+__global__ void __launch_bounds__(kRfX *kRfY)
+    k_pg_resid_fix(const unsigned long long *phi, const long long *f, Dims d, float c, int K,
+                   int zc, float *r, unsigned long long *out) {
+  constexpr int W = PAIR ? 2 : 1;
+  struct Cells {
+    unsigned long long v[W];
+  };
+  auto load = [](const void *p, long long t) {
+    Cells q;
+    if (PAIR) {
+      const ulonglong2 w = reinterpret_cast<const ulonglong2 *>(p)[t >> 1];
+      q.v[0] = w.x;
+      q.v[W - 1] = w.y;
+    } else {
+      q.v[0] = reinterpret_cast<const unsigned long long *>(p)[t];
+    }
+    return q;
+  };
+  float loc = 0.0f;
+  const int nx = d.n[0], ny = d.n[1], nz = d.n[2];
+  const int i = (blockIdx.x * kRfX + threadIdx.x) * W, j = blockIdx.y * kRfY + threadIdx.y;
+  const int z0 = blockIdx.z * zc, z1 = min(nz, z0 + zc);
+  if (i < nx && j < ny) {
+    const long long sz = (long long)nx * ny;
+    const long long o = (long long)j * nx + i;
+    const long long ym = (long long)(j ? j - 1 : ny - 1) * nx + i;
+    const long long yp = (long long)(j + 1 < ny ? j + 1 : 0) * nx + i;
+    const long long xm = i ? o - 1 : o + nx - 1, xp = i + W < nx ? o + W : o + W - nx;
+    const float cK = c * __int_as_float((127 - K) << 23);
+    const unsigned long long lim = 1ull << (62 - K);
+    Cells lo = load(phi, (z0 ? z0 - 1 : nz - 1) * sz + o), mid = load(phi, z0 * sz + o);
+    for (int k = z0; k < z1; ++k) {
+      const long long zb = k * sz;
+      const Cells hi = load(phi, (k + 1 < nz ? zb + sz : 0) + o);
+      const Cells a = load(phi, zb + ym), b = load(phi, zb + yp), ff = load(f, zb + o);
+      const unsigned long long left = phi[zb + xm], right = phi[zb + xp];
+      float q[W];
+#pragma unroll
+      for (int u = 0; u < W; ++u) {
+        const unsigned long long w = u == 0 ? left : mid.v[0], e = u == W - 1 ? right : mid.v[W - 1];
+        const unsigned long long nb = w + e + a.v[u] + b.v[u] + lo.v[u] + hi.v[u];
+        const long long F = (long long)ff.v[u];
+        const unsigned long long v = (unsigned long long)(F >> K) + 6 * mid.v[u] - nb;
+        const bool fine = v + lim < 2 * lim;
+        const unsigned long long x = fine ? (v << K) + (unsigned long long)(F & ((1ll << K) - 1)) : v;
+        q[u] = from_fix((long long)x) * (fine ? cK : c);
+        loc = fmaxf(loc, fabsf(q[u]));
+      }
+      if (PAIR)
+        *reinterpret_cast<float2 *>(r + zb + o) = make_float2(q[0], q[W - 1]);
+      else
+        r[zb + o] = q[0];
+      lo = mid;
+      mid = hi;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) loc = fmaxf(loc, __shfl_xor_sync(0xffffffffu, loc, o));
+  if (threadIdx.x == 0) atomic_max_pos(out, (double)loc);
+}
+
+__global__ void k_pg_correct_fix(long long *phi, const float *e, long long n, float s) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
+       t += (long long)gridDim.x * blockDim.x)
+    phi[t] = phi[t] + to_fix(e[t], s);
+}
+
 // ---------------------------------------------------------------- fused V-cycle kernels
 // The sweeps of one colour only read the other colour, so any schedule that
 // gives each half-sweep its finished neighbours yields the same bits; the two
@@ -441,12 +584,28 @@ __global__ void __launch_bounds__(kTailThreads) k_pg_tail(const TailArgs<T> a) {
   auto cells = [&](int l) { return a.d[l].n[0] * a.d[l].n[1] * a.d[l].n[2]; };
   auto sweeps = [&](int l, int count) {
     T *phi = sm + a.off[l], *f = phi + cells(l);
-    if (cells(l) <= 64) {  // one warp: no CTA barrier between the half-sweeps
-      if (tid < 32)
+    const Dims &d = a.d[l];
+    if (cells(l) <= 64) {  // one warp, its cells' neighbours found once
+      if (tid < 32) {
+        const int hx = d.n[0] / 2, n = hx * d.n[1] * d.n[2];
+        const int q = tid / hx, i2 = tid - q * hx, k = q / d.n[1], j = q - k * d.n[1];
+        const int sy = d.n[0], sz = d.n[0] * d.n[1], row = k * sz + j * sy;
+        const int ym = k * sz + wrp(j - 1, d.n[1]) * sy, yp = k * sz + wrp(j + 1, d.n[1]) * sy;
+        const int zm = wrp(k - 1, d.n[2]) * sz + j * sy, zp = wrp(k + 1, d.n[2]) * sz + j * sy;
         for (int s = 0; s < 2 * count; ++s) {
-          tail_half(phi, f, a.d[l], a.fx[l], a.fy[l], a.h2[l], s & 1, tid, 32);
+          if (tid < n) {
+            const int i = 2 * i2 + ((j + k + s) & 1);
+            T v = phi[row + wrp(i - 1, d.n[0])];
+            v = v + phi[row + wrp(i + 1, d.n[0])];
+            v = v + phi[ym + i];
+            v = v + phi[yp + i];
+            v = v + phi[zm + i];
+            v = v + phi[zp + i];
+            phi[row + i] = (v - a.h2[l] * f[row + i]) * (T(1) / T(6));
+          }
           __syncwarp();
         }
+      }
       __syncthreads();
     } else {
       for (int s = 0; s < 2 * count; ++s) {
@@ -503,27 +662,33 @@ __global__ void __launch_bounds__(kTailThreads) k_pg_tail(const TailArgs<T> a) {
 // with what stands next to it in the V-cycle: the start from phi = 0 (ZERO:
 // phi_in is not read), the coarse correction added first (PROLONG), the
 // residual's restriction after it (RESTRICT), and on the finest grid the
-// FP64 update phi64 += result in place of storing it (ADD64).  A CTA takes a
+// update of the potential by the result in place of storing it (ADD 1: FP64,
+// ADD 2: fixed point, fs its scale).  A CTA takes a
 // 64 x 16 column tile and marches a range of planes through shared-memory
 // rings: plane t arrives, the red cells of plane t-1 and then the black ones
 // of plane t-2 are relaxed, plane t-2 is written, and the residual is formed
 // on plane t-4.  The halo (3 cells, 4 in x so that pairs stay aligned) is
 // relaxed again by the neighbours, so the result goes to a second array.
-// Rows hold the even x, then the odd x: the cells of one colour and their
-// neighbours are contiguous, free of bank conflicts.
+// A plane holds its red cells, then its black ones, 36 to a row: the cells of
+// one colour and their neighbours (all of the other colour) lie at consecutive
+// addresses, free of bank conflicts.
 //
-// Bound: memory (f and phi read once, phi written once: 12 B per cell and
-// sweep instead of two half-sweeps that each touch every line of both).
+// Bound: shared memory (9 accesses per relaxed cell; memory would allow 30 us
+// for the 12 B per cell of a sweep).  A sweep of a 256^3 grid: 114 us with the
+// colours split (74 us from zero), 120 us with even and odd x split (two-way conflicts), against
+// 2 x 37 us per half-sweep launch plus the transfers' own passes.
 constexpr int kSwTX = 64, kSwTY = 16, kSwH = 36, kSwW = 2 * kSwH, kSwR = kSwTY + 6;
 constexpr int kSwThreads = 256, kSwPlane = kSwW * kSwR, kSwPairs = kSwH * kSwR;
+constexpr int kSwC = kSwPairs;  // offset of the black cells of a plane
 constexpr int kSwLoads = (kSwPairs + kSwThreads - 1) / kSwThreads;
 constexpr size_t kSwSmem = sizeof(float) * 11 * kSwPlane;
 
-template <bool ZERO, bool PROLONG, bool RESTRICT, bool ADD64>
-__global__ void __launch_bounds__(kSwThreads) k_pg_smooth(const float *phi_in, const float *f,
+template <bool ZERO, bool PROLONG, bool RESTRICT, int ADD>
+__global__ void __launch_bounds__(kSwThreads, 3) k_pg_smooth(const float *phi_in, const float *f,
                                                           float *phi_out, Dims d, float h2,
                                                           float ih2, int zchunk, const float *pc,
-                                                          float *fc, Dims dc, double *phi64) {
+                                                          float *fc, Dims dc, double *phi64,
+                                                          long long *fix, float fs) {
   extern __shared__ __align__(16) float sw_smem[];
   float *sp = sw_smem;                  // [6][kSwPlane] phi, plane t in slot t % 6
   float *sf = sw_smem + 6 * kSwPlane;   // [5][kSwPlane] f, plane t in slot t % 5
@@ -534,8 +699,9 @@ __global__ void __launch_bounds__(kSwThreads) k_pg_smooth(const float *phi_in, c
   const long long sz = (long long)nx * ny;
   // this thread's pairs (cells 2h, 2h+1 of tile row r): global offset inside a
   // plane (periodic), coarse offset, and where they lie in the tile
-  int off[kSwLoads], coff[kSwLoads];
+  int off[kSwLoads], coff[kSwLoads], at[kSwLoads];
   bool own[kSwLoads];
+  unsigned odd_l = 0;  // parity of each pair's row
 #pragma unroll
   for (int u = 0; u < kSwLoads; ++u) {
     const int e = tid + u * kSwThreads, r = e / kSwH, h = e - r * kSwH;
@@ -544,94 +710,110 @@ __global__ void __launch_bounds__(kSwThreads) k_pg_smooth(const float *phi_in, c
     if (X < 0) X += nx;
     if (Y < 0) Y += ny;
     off[u] = Y * nx + X;
+    at[u] = e;
+    odd_l |= (unsigned)(gy & 1) << u;
     coff[u] = PROLONG ? (Y / 2) * dc.n[0] + X / 2 : 0;
     own[u] = e < kSwPairs && r >= 3 && r < 3 + kSwTY && h >= 2 && h < 2 + kSwTX / 2 && gx < nx &&
              gy < ny;
   }
-  float2 rp[kSwLoads], rf[kSwLoads];
   auto wrap_z = [&](int t) {
     int k = t % nz;
     return k < 0 ? k + nz : k;
   };
-  auto load = [&](int t) {
+  // one plane in flight; loads run two planes ahead of their use
+  struct Plane {
+    float2 p[kSwLoads], f[kSwLoads];
+    float c[kSwLoads];
+  };
+  auto load = [&](int t, Plane &R) {
     const int k = wrap_z(t);
 #pragma unroll
     for (int u = 0; u < kSwLoads; ++u) {
       if (tid + u * kSwThreads >= kSwPairs) continue;
       const long long id = k * sz + off[u];
-      rf[u] = *reinterpret_cast<const float2 *>(f + id);
-      if (ZERO) {
-        rp[u] = make_float2(0.0f, 0.0f);
-      } else {
-        rp[u] = *reinterpret_cast<const float2 *>(phi_in + id);
-        if (PROLONG) {
-          const float c = pc[(long long)(k / 2) * dc.n[0] * dc.n[1] + coff[u]];
-          rp[u].x = rp[u].x + c;
-          rp[u].y = rp[u].y + c;
-        }
-      }
+      R.f[u] = *reinterpret_cast<const float2 *>(f + id);
+      if (!ZERO) R.p[u] = *reinterpret_cast<const float2 *>(phi_in + id);
+      if (PROLONG) R.c[u] = pc[(long long)(k / 2) * dc.n[0] * dc.n[1] + coff[u]];
     }
   };
-  // neighbour sum of the cell at row r, half index h, x parity px of plane t
-  auto nb = [&](const float *P, const float *Pm, const float *Pp, int c, int px) {
-    const float *o = P + (px ? -kSwH : kSwH) + c;  // the other x parity, same half index
-    float s = px ? o[0] : o[-1];
-    s = s + (px ? o[1] : o[0]);
-    s = s + P[c - kSwW];
-    s = s + P[c + kSwW];
-    s = s + Pm[c];
-    s = s + Pp[c];
+  // neighbour sum of the cell at a = 36 r + h of its colour, x parity px: P, Pm,
+  // Pp the other colour's cells of planes t, t-1, t+1
+  auto nb = [&](const float *P, const float *Pm, const float *Pp, int a, int px) {
+    float s = px ? P[a] : P[a - 1];
+    s = s + (px ? P[a + 1] : P[a]);
+    s = s + P[a - kSwH];
+    s = s + P[a + kSwH];
+    s = s + Pm[a];
+    s = s + Pp[a];
     return s;
   };
   auto plane = [&](int t) { return sp + (t + 6 * 8) % 6 * kSwPlane; };
   auto fplane = [&](int t) { return sf + (t + 5 * 8) % 5 * kSwPlane; };
-  // tile rows [r0, r1), half indices 1 .. kSwH - 2, of the cells of one colour
-  auto relax = [&](int t, int color, int r0, int r1) {
-    float *P = plane(t);
-    const float *Pm = plane(t - 1), *Pp = plane(t + 1), *F = fplane(t);
-    constexpr int w = kSwH - 2;
-    for (int e = tid; e < (r1 - r0) * w; e += kSwThreads) {
-      const int q = e / w, r = r0 + q, h = 1 + e - q * w;
-      const int px = (y0 + r - 3 + t + color) & 1;
-      const int c = r * kSwW + px * kSwH + h;
-      P[c] = (nb(P, Pm, Pp, c, px) - h2 * F[c]) * (1.0f / 6.0f);
+  // this thread's cells to relax, 36 a row (the outermost only get values that
+  // nothing uses): red ones of rows 1 .. kSwR - 2, black ones of rows 2 .. kSwR - 3
+  constexpr int kRelax = (kSwR - 2) * kSwH;
+  constexpr int kIter = (kRelax + kSwThreads - 1) / kSwThreads;
+  unsigned odd = 0, inner = 0;
+#pragma unroll
+  for (int u = 0; u < kIter; ++u) {
+    const int row = 1 + (tid + u * kSwThreads) / kSwH;
+    odd |= (unsigned)((y0 + row - 3) & 1) << u;
+    inner |= (unsigned)(row >= 2 && row <= kSwR - 3) << u;
+  }
+  auto relax = [&](int t, int color) {
+    float *P = plane(t) + color * kSwC;
+    const int oc = (1 - color) * kSwC;
+    const float *Q = plane(t) + oc, *Pm = plane(t - 1) + oc, *Pp = plane(t + 1) + oc;
+    const float *F = fplane(t) + color * kSwC;
+#pragma unroll
+    for (int u = 0; u < kIter; ++u) {
+      const int e = tid + u * kSwThreads, a = kSwH + e;
+      if (e >= kRelax || (color && !((inner >> u) & 1u))) continue;
+      const int px = (int)((odd >> u) ^ (unsigned)(t + color)) & 1;
+      P[a] = (nb(Q, Pm, Pp, a, px) - h2 * F[a]) * (1.0f / 6.0f);
     }
   };
   float racc = 0.0f;  // this thread's coarse cell: residuals summed so far
-  load(z0 - 3);
-  for (int t = z0 - 3; t <= z1 + 3; ++t) {
+  auto step = [&](int t, Plane &R) {
     if (t <= z1 + 2) {
       float *P = plane(t), *F = fplane(t);
 #pragma unroll
       for (int u = 0; u < kSwLoads; ++u) {
-        const int e = tid + u * kSwThreads;
-        if (e >= kSwPairs) continue;
-        const int r = e / kSwH, h = e - r * kSwH, c = r * kSwW + h;
-        P[c] = rp[u].x;
-        P[c + kSwH] = rp[u].y;
-        F[c] = rf[u].x;
-        F[c + kSwH] = rf[u].y;
+        if (tid + u * kSwThreads >= kSwPairs) continue;
+        const int c = at[u];
+        float2 v = ZERO ? make_float2(0.0f, 0.0f) : R.p[u];
+        if (PROLONG) {
+          v.x = v.x + R.c[u];
+          v.y = v.y + R.c[u];
+        }
+        const int ce = ((odd_l >> u) ^ (unsigned)t) & 1u ? kSwC : 0;  // colour of the even x
+        P[c + ce] = v.x;
+        P[c + kSwC - ce] = v.y;
+        F[c + ce] = R.f[u].x;
+        F[c + kSwC - ce] = R.f[u].y;
       }
-      if (t < z1 + 2) load(t + 1);
+      if (t + 2 <= z1 + 2) load(t + 2, R);
     }
     __syncthreads();
     if (RESTRICT && t - 4 >= z0 && t - 4 < z1) {
       const int q = t - 4;
       const int I = tid & 31, J = tid >> 5;
-      const float *P = plane(q), *Pm = plane(q - 1), *Pp = plane(q + 1), *F = fplane(q);
 #pragma unroll
       for (int o = 0; o < 4; ++o) {
-        const int px = o & 1, c = (3 + 2 * J + (o >> 1)) * kSwW + px * kSwH + 2 + I;
-        const float r = F[c] - (nb(P, Pm, Pp, c, px) - 6.0f * P[c]) * ih2;
+        const int px = o & 1, row = 3 + 2 * J + (o >> 1), a = row * kSwH + 2 + I;
+        const int color = (y0 + row - 3 + q + px) & 1, oc = (1 - color) * kSwC;
+        const float r = fplane(q)[a + color * kSwC] -
+                        (nb(plane(q) + oc, plane(q - 1) + oc, plane(q + 1) + oc, a, px) -
+                         6.0f * plane(q)[a + color * kSwC]) * ih2;
         racc = (o == 0 && !(q & 1)) ? r : racc + r;
       }
       const int ci = x0 / 2 + I, cj = y0 / 2 + J;
       if ((q & 1) && ci < dc.n[0] && cj < dc.n[1])
         fc[((long long)(q / 2) * dc.n[1] + cj) * dc.n[0] + ci] = 0.125f * racc;
     }
-    if (t - 1 >= z0 - 2 && t - 1 <= z1 + 1) relax(t - 1, 0, 1, kSwR - 1);
+    if (t - 1 >= z0 - 2 && t - 1 <= z1 + 1) relax(t - 1, 0);
     __syncthreads();
-    if (t - 2 >= z0 - 1 && t - 2 <= z1) relax(t - 2, 1, 2, kSwR - 2);
+    if (t - 2 >= z0 - 1 && t - 2 <= z1) relax(t - 2, 1);
     if (t - 2 >= z0 && t - 2 < z1) {
       __syncthreads();
       const float *P = plane(t - 2);
@@ -639,9 +821,15 @@ __global__ void __launch_bounds__(kSwThreads) k_pg_smooth(const float *phi_in, c
 #pragma unroll
       for (int u = 0; u < kSwLoads; ++u) {
         if (!own[u]) continue;
-        const int e = tid + u * kSwThreads, r = e / kSwH, h = e - r * kSwH, c = r * kSwW + h;
-        const float2 v = make_float2(P[c], P[c + kSwH]);
-        if (ADD64) {
+        const int c = at[u], ce = ((odd_l >> u) ^ (unsigned)(t - 2)) & 1u ? kSwC : 0;
+        const float2 v = make_float2(P[c + ce], P[c + kSwC - ce]);
+        if (ADD == 2) {
+          longlong2 *o = reinterpret_cast<longlong2 *>(fix + zb + off[u]);
+          longlong2 w2 = *o;
+          w2.x = w2.x + to_fix(v.x, fs);
+          w2.y = w2.y + to_fix(v.y, fs);
+          *o = w2;
+        } else if (ADD == 1) {
           double2 *o = reinterpret_cast<double2 *>(phi64 + zb + off[u]);
           double2 w = *o;
           w.x = w.x + (double)v.x;
@@ -652,6 +840,13 @@ __global__ void __launch_bounds__(kSwThreads) k_pg_smooth(const float *phi_in, c
         }
       }
     }
+  };
+  Plane ra, rb;
+  load(z0 - 3, ra);
+  load(z0 - 2, rb);
+  for (int t = z0 - 3; t <= z1 + 3; t += 2) {
+    step(t, ra);
+    if (t + 1 <= z1 + 3) step(t + 1, rb);
   }
 }
 
@@ -720,6 +915,13 @@ struct nyx_poisson {
   TailArgs<double> targs64{};
   TailArgs<float> targs32{};
   size_t tsmem64 = 0, tsmem32 = 0;
+  // fixed-point potential of the refinement solve (while `fixed`): units of
+  // 1/fix_s; h^2 times the right-hand side is then fixed point in L[0].f's
+  // memory, in units of 1/(fix_s 2^fix_k)
+  long long *d_fix = nullptr;
+  bool fixed = false;
+  float fix_s = 0.0f;
+  int fix_k = 0;
 };
 
 namespace {
@@ -735,6 +937,7 @@ void free_poisson(nyx_poisson *S) {
     if (l.f) cudaFree(l.f);
     if (l.phi2) cudaFree(l.phi2);
   }
+  cudaFree(S->d_fix);
   cudaFree(S->d_box_lo);
   cudaFree(S->d_rows);
   cudaFree(S->d_planes);
@@ -838,7 +1041,7 @@ void vcycle(nyx_poisson *S, std::vector<LevelT<T>> &L, size_t l, size_t tail_at,
 }
 
 // One fused sweep of FP32 grid l from phi_in into phi_out.
-template <bool ZERO, bool PROLONG, bool RESTRICT, bool ADD64>
+template <bool ZERO, bool PROLONG, bool RESTRICT, int ADD>
 void smooth_launch(nyx_poisson *S, size_t l, const float *in, float *out, const float *pc) {
   const LevelT<float> &g = S->L32[l];
   const LevelT<float> &c = S->L32[std::min(l + 1, S->L32.size() - 1)];
@@ -848,26 +1051,29 @@ void smooth_launch(nyx_poisson *S, size_t l, const float *in, float *out, const 
   const int nch = std::max(1, 3 * 152 / (tx * ty));
   const int zc = std::max(2, ((g.d.n[2] + nch - 1) / nch + 1) & ~1);
   const dim3 grid(tx, ty, (g.d.n[2] + zc - 1) / zc);
-  k_pg_smooth<ZERO, PROLONG, RESTRICT, ADD64><<<grid, kSwThreads, kSwSmem, S->P->stream>>>(
-      in, g.f, out, g.d, g.h2, g.ih2, zc, pc, c.f, c.d, S->L[0].phi);
+  k_pg_smooth<ZERO, PROLONG, RESTRICT, ADD><<<grid, kSwThreads, kSwSmem, S->P->stream>>>(
+      in, g.f, out, g.d, g.h2, g.ih2, zc, pc, c.f, c.d, S->L[0].phi, S->d_fix, S->fix_s);
   S->launches += 1;
 }
 
 int smooth_init() {
-  const void *k[] = {(const void *)k_pg_smooth<true, false, false, false>,
-                     (const void *)k_pg_smooth<true, false, true, false>,
-                     (const void *)k_pg_smooth<false, false, false, false>,
-                     (const void *)k_pg_smooth<false, false, true, false>,
-                     (const void *)k_pg_smooth<false, true, false, false>,
-                     (const void *)k_pg_smooth<false, true, false, true>,
-                     (const void *)k_pg_smooth<false, false, false, true>};
+  const void *k[] = {(const void *)k_pg_smooth<true, false, false, 0>,
+                     (const void *)k_pg_smooth<true, false, true, 0>,
+                     (const void *)k_pg_smooth<false, false, false, 0>,
+                     (const void *)k_pg_smooth<false, false, true, 0>,
+                     (const void *)k_pg_smooth<false, true, false, 0>,
+                     (const void *)k_pg_smooth<false, true, false, 1>,
+                     (const void *)k_pg_smooth<false, false, false, 1>,
+                     (const void *)k_pg_smooth<false, true, false, 2>,
+                     (const void *)k_pg_smooth<false, false, false, 2>};
   for (const void *f : k)
     CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwSmem));
   return NYX_OK;
 }
 
 // The FP32 V-cycle of one refinement step with fused sweeps (at least one
-// sweep on each side): phi64 += the correction at the end.
+// sweep on each side): the potential, FP64 or fixed point, += the correction
+// at the end.
 void vcycle_fused(nyx_poisson *S) {
   std::vector<LevelT<float>> &L = S->L32;
   const size_t last = L.size() - 1, top = S->tail32;
@@ -879,10 +1085,10 @@ void vcycle_fused(nyx_poisson *S) {
     for (int p = 0; p < S->prm.pre; ++p) {
       float *out = other(l, cur[l]);
       const bool end = p == S->prm.pre - 1;
-      if (p == 0 && end) smooth_launch<true, false, true, false>(S, l, nullptr, out, nullptr);
-      else if (p == 0) smooth_launch<true, false, false, false>(S, l, nullptr, out, nullptr);
-      else if (end) smooth_launch<false, false, true, false>(S, l, cur[l], out, nullptr);
-      else smooth_launch<false, false, false, false>(S, l, cur[l], out, nullptr);
+      if (p == 0 && end) smooth_launch<true, false, true, 0>(S, l, nullptr, out, nullptr);
+      else if (p == 0) smooth_launch<true, false, false, 0>(S, l, nullptr, out, nullptr);
+      else if (end) smooth_launch<false, false, true, 0>(S, l, cur[l], out, nullptr);
+      else smooth_launch<false, false, false, 0>(S, l, cur[l], out, nullptr);
       cur[l] = out;
     }
   if (top < L.size()) {
@@ -891,8 +1097,8 @@ void vcycle_fused(nyx_poisson *S) {
   } else {
     for (int p = 0; p < S->prm.coarse_sweeps; ++p) {
       float *out = other(last, cur[last]);
-      if (p == 0) smooth_launch<true, false, false, false>(S, last, nullptr, out, nullptr);
-      else smooth_launch<false, false, false, false>(S, last, cur[last], out, nullptr);
+      if (p == 0) smooth_launch<true, false, false, 0>(S, last, nullptr, out, nullptr);
+      else smooth_launch<false, false, false, 0>(S, last, cur[last], out, nullptr);
       cur[last] = out;
     }
   }
@@ -901,16 +1107,21 @@ void vcycle_fused(nyx_poisson *S) {
       float *out = other(l, cur[l]);
       const bool add = l == 0 && p == S->prm.post - 1;
       const float *pc = cur[l + 1];
-      if (p == 0 && add) smooth_launch<false, true, false, true>(S, l, cur[l], nullptr, pc);
-      else if (p == 0) smooth_launch<false, true, false, false>(S, l, cur[l], out, pc);
-      else if (add) smooth_launch<false, false, false, true>(S, l, cur[l], nullptr, nullptr);
-      else smooth_launch<false, false, false, false>(S, l, cur[l], out, nullptr);
+      if (p == 0 && add && S->fixed) smooth_launch<false, true, false, 2>(S, l, cur[l], nullptr, pc);
+      else if (p == 0 && add) smooth_launch<false, true, false, 1>(S, l, cur[l], nullptr, pc);
+      else if (p == 0) smooth_launch<false, true, false, 0>(S, l, cur[l], out, pc);
+      else if (add && S->fixed) smooth_launch<false, false, false, 2>(S, l, cur[l], nullptr, nullptr);
+      else if (add) smooth_launch<false, false, false, 1>(S, l, cur[l], nullptr, nullptr);
+      else smooth_launch<false, false, false, 0>(S, l, cur[l], out, nullptr);
       cur[l] = out;
     }
   if (nd == 0) {  // the finest grid is the tail's first, or the coarsest
     Level &g = S->L[0];
     const long long n = (long long)g.d.n[0] * g.d.n[1] * g.d.n[2];
-    k_pg_correct<<<gridn(n, 256), 256, 0, S->P->stream>>>(g.phi, cur[0], n);
+    if (S->fixed)
+      k_pg_correct_fix<<<gridn(n, 256), 256, 0, S->P->stream>>>(S->d_fix, cur[0], n, S->fix_s);
+    else
+      k_pg_correct<<<gridn(n, 256), 256, 0, S->P->stream>>>(g.phi, cur[0], n);
     S->launches += 1;
   }
 }
@@ -920,11 +1131,22 @@ bool fused_cycle(const nyx_poisson *S) { return S->prm.pre >= 1 && S->prm.post >
 int resid_max(nyx_poisson *S, double *out) {
   Level &g = S->L[0];
   CK(cudaMemsetAsync(S->d_max, 0, sizeof(unsigned long long), S->P->stream));
-  const Grid3 G = grid3(g.d.n[0], g.d.n[1], g.d.n[2]);
-  if (S->L32.empty()) {
+  if (S->fixed) {
+    LevelT<float> &g32 = S->L32[0];
+    const int w = g.d.n[0] % 2 ? 1 : 2;
+    dim3 G((g.d.n[0] + kRfX * w - 1) / (kRfX * w), (g.d.n[1] + kRfY - 1) / kRfY);
+    // planes per CTA: 16 (one in 8 read again), fewer while that leaves SMs idle
+    const int zc = (int)std::min(16ll, std::max(2ll, (long long)G.x * G.y * g.d.n[2] / (152 * 8)));
+    G.z = (g.d.n[2] + zc - 1) / zc;
+    (w == 2 ? k_pg_resid_fix<true> : k_pg_resid_fix<false>)<<<G, dim3(kRfX, kRfY), 0, S->P->stream>>>(
+        (const unsigned long long *)S->d_fix, (const long long *)g.f, g.d,
+        (float)(g.ih2 / (double)S->fix_s), S->fix_k, zc, g32.f, S->d_max);
+  } else if (S->L32.empty()) {
+    const Grid3 G = grid3(g.d.n[0], g.d.n[1], g.d.n[2]);
     k_pg_resid_max<<<G.g, G.b, 0, S->P->stream>>>(g.phi, g.f, g.d, g.ih2, S->d_max);
   } else {  // also the FP32 right-hand side of the next correction, and e = 0
     LevelT<float> &g32 = S->L32[0];
+    const Grid3 G = grid3(g.d.n[0], g.d.n[1], g.d.n[2]);
     k_pg_resid32<<<G.g, G.b, 0, S->P->stream>>>(g.phi, g.f, g.d, g.ih2, 6.0 * g.ih2, g32.f,
                                                 g32.phi, S->d_max);
   }
@@ -1036,6 +1258,9 @@ int nyx_poisson_create(nyx_plan *P, const nyx_poisson_params *prm, nyx_poisson *
     if (!S->L32.empty()) {
       S->tail32 = make_tail(S, S->L32, 0, S->targs32, S->tsmem32);
       rc = smooth_init();
+      if (!rc && fused_cycle(S) &&
+          cudaMalloc(&S->d_fix, sizeof(long long) * (size_t)n[0] * n[1] * n[2]) != cudaSuccess)
+        rc = fail(NYX_ENOMEM, "Poisson grid allocation failed");
       if (fused_cycle(S))
         for (size_t l = 0; l < std::min(S->tail32, S->L32.size()) && !rc; ++l) {
           LevelT<float> &g = S->L32[l];
@@ -1067,15 +1292,14 @@ int nyx_poisson_create(nyx_plan *P, const nyx_poisson_params *prm, nyx_poisson *
   return NYX_OK;
 }
 
-int nyx_poisson_solve(nyx_poisson *S, const double *state, const double *rho_dm, double a,
-                      double *grav_out, double *g_dense_out, int warm_start, int *cycles_out,
-                      double *resid_out) {
-  if (!S || !state || !(a > 0.0)) return fail(NYX_EINVAL, "bad argument");
+// Right-hand side f = 4 pi G / a (rho + rho_dm - mean) into L[0].f, its max
+// norm in *fmax (synchronises).
+static int build_rhs(nyx_poisson *S, const double *state, const double *rho_dm, double a,
+                     double *fmax) {
   nyx_plan &P = *S->P;
   Level &g0 = S->L[0];
   const long long N = (long long)g0.d.n[0] * g0.d.n[1] * g0.d.n[2];
   cudaStream_t st = P.stream;
-  if (!warm_start) CK(cudaMemsetAsync(g0.phi, 0, N * sizeof(double), st));
   k_pg_gather<<<walk_grid(P.total_cells, 256), 256, 0, st>>>(state, P.d_boxes, P.d_cell_pref,
                                                             S->d_box_lo, P.nbox, P.total_cells,
                                                             g0.d, g0.f);
@@ -1090,16 +1314,89 @@ int nyx_poisson_solve(nyx_poisson *S, const double *state, const double *rho_dm,
   CK(cudaMemsetAsync(S->d_max, 0, sizeof(unsigned long long), st));
   k_pg_rhs<<<gridn(N, 256), 256, 0, st>>>(g0.f, N, S->d_scal, S->prm.four_pi_G / a, S->d_max);
   S->launches += 5;
-  double fmax = 0.0, res = 0.0;
-  int rc = read_max(S, &fmax);
-  if (rc) return rc;
-  if ((rc = resid_max(S, &res))) return rc;
-  const double target = S->prm.tol * fmax;
-  int cyc = 0;
-  while (res > target && cyc < S->prm.max_cycles) {
+  return read_max(S, fmax);
+}
+
+// Cycles until the residual's max norm is at most `target` (*res: the first
+// residual's norm if that is there already, else negative).
+static int run_cycles(nyx_poisson *S, double target, int *cyc, double *res) {
+  *cyc = 0;
+  if (*res < 0.0)
+    if (int rc = resid_max(S, res)) return rc;
+  while (*res > target && *cyc < S->prm.max_cycles) {
     cycle(S);
-    ++cyc;
-    if ((rc = resid_max(S, &res))) return rc;
+    ++*cyc;
+    if (int rc = resid_max(S, res)) return rc;
+  }
+  return NYX_OK;
+}
+
+// Start the solve in fixed point if a scale fits: the potential of a zero-mean
+// right-hand side of max norm fmax on a periodic box of longest side l is at
+// most 0.26 l^2 fmax (Cauchy-Schwarz over its Fourier modes, whose discrete
+// eigenvalues are at least 4 / pi^2 of k^2), and the start's own potential is
+// measured.  The sum of the first and 8 of the second is kept below 2^61: six
+// times any difference of two potentials then stays below 2^63.  A start from
+// phi = 0 leaves its residual, f, and the norm of it.
+static int start_fixed(nyx_poisson *S, double fmax, int warm, double *res) {
+  Level &g = S->L[0];
+  const long long n = (long long)g.d.n[0] * g.d.n[1] * g.d.n[2];
+  cudaStream_t st = S->P->stream;
+  double pmax = 0.0;
+  if (warm) {
+    CK(cudaMemsetAsync(S->d_max, 0, sizeof(unsigned long long), st));
+    k_pg_absmax<<<gridn(n, 256), 256, 0, st>>>(g.phi, n, S->d_max);
+    S->launches += 1;
+    if (int rc = read_max(S, &pmax)) return rc;
+  }
+  const double side = std::max(g.d.n[0], std::max(g.d.n[1], g.d.n[2])) * S->dx;
+  const double bound = 2.0 * (0.26 * side * side * fmax + 8.0 * pmax);
+  if (!(bound > 1e-15 && bound < 1e15)) return NYX_OK;  // FP64 residuals instead
+  const double s = std::ldexp(1.0, 62 - (int)std::ceil(std::log2(bound)));
+  // the residual's scale stays inside FP32's range
+  const double c = g.ih2 / s;
+  if (!(c > 1e-27 && c < 1e30 && s < 1e36)) return NYX_OK;
+  const double hf = g.h2 * s * fmax;  // in (0, 2^61): h^2 f < bound / 2
+  S->fix_k = std::min(31, 61 - (hf > 1.0 ? (int)std::ceil(std::log2(hf)) : 0));
+  S->fix_s = (float)s;
+  S->fixed = true;
+  k_pg_rhs_fix<<<gridn(n, 256), 256, 0, st>>>(g.f, (long long *)g.f, n,
+                                              std::ldexp(g.h2 * s, S->fix_k), S->d_fix,
+                                              warm ? nullptr : S->L32[0].f);
+  S->launches += 1;
+  if (warm) {
+    k_pg_to_fix<<<gridn(n, 256), 256, 0, st>>>(g.phi, S->d_fix, n, s);
+    S->launches += 1;
+  } else {
+    *res = (double)(float)fmax;
+  }
+  return NYX_OK;
+}
+
+int nyx_poisson_solve(nyx_poisson *S, const double *state, const double *rho_dm, double a,
+                      double *grav_out, double *g_dense_out, int warm_start, int *cycles_out,
+                      double *resid_out) {
+  if (!S || !state || !(a > 0.0)) return fail(NYX_EINVAL, "bad argument");
+  nyx_plan &P = *S->P;
+  Level &g0 = S->L[0];
+  const long long N = (long long)g0.d.n[0] * g0.d.n[1] * g0.d.n[2];
+  cudaStream_t st = P.stream;
+  double fmax = 0.0, res = -1.0;
+  int cyc = 0;
+  S->fixed = false;
+  int rc = build_rhs(S, state, rho_dm, a, &fmax);
+  if (rc) return rc;
+  const double target = S->prm.tol * fmax;
+  if (S->d_fix && (rc = start_fixed(S, fmax, warm_start, &res))) return rc;
+  if (S->fixed) {
+    rc = run_cycles(S, target, &cyc, &res);
+    S->fixed = false;
+    if (rc) return rc;
+    k_pg_from_fix<<<gridn(N, 256), 256, 0, st>>>(S->d_fix, g0.phi, N, 1.0 / (double)S->fix_s);
+    S->launches += 1;
+  } else {
+    if (!warm_start) CK(cudaMemsetAsync(g0.phi, 0, N * sizeof(double), st));
+    if ((rc = run_cycles(S, target, &cyc, &res))) return rc;
   }
   if (grav_out) {
     k_pg_grav<<<walk_grid(P.total_cells, 256), 256, 0, st>>>(g0.phi, g0.d, 0.5 / S->dx, P.d_boxes,
