@@ -217,7 +217,37 @@ bool build_fill(const nyx_plan &P, std::vector<FillRect> out[4]) {
   return true;
 }
 
-int upload_pass(FillPass &p, const std::vector<FillRect> &rects) {
+// The fill kernel gives a CTA a rectangle: cut them (in z, then y; rows stay
+// whole) to 4096 cells, and to fewer on small levels, so that a level of few
+// boxes gives every SM work.  The 26 rectangles of one 192^3 box: 304 us whole,
+// 25 us cut; of one 32^3 box 11.5 and 4.6 us.
+std::vector<FillRect> cut_rects(const std::vector<FillRect> &rects) {
+  long long total = 0;
+  for (const FillRect &R : rects) total += (long long)R.ext[0] * R.ext[1] * R.ext[2];
+  const long long lim = std::min(4096ll, std::max(512ll, total / (152 * 8)));
+  std::vector<FillRect> out;
+  out.reserve(rects.size());
+  for (const FillRect &R : rects) {
+    const long long row = R.ext[0];
+    const int sy = (int)std::max(1ll, std::min((long long)R.ext[1], lim / row));
+    const int sz = (int)std::max(1ll, std::min((long long)R.ext[2], lim / (row * sy)));
+    for (int z = 0; z < R.ext[2]; z += sz)
+      for (int y = 0; y < R.ext[1]; y += sy) {
+        FillRect Q = R;
+        Q.dlo[1] += y;
+        Q.slo[1] += R.sstep[1] * y;
+        Q.ext[1] = std::min(sy, R.ext[1] - y);
+        Q.dlo[2] += z;
+        Q.slo[2] += R.sstep[2] * z;
+        Q.ext[2] = std::min(sz, R.ext[2] - z);
+        out.push_back(Q);
+      }
+  }
+  return out;
+}
+
+int upload_pass(FillPass &p, const std::vector<FillRect> &whole) {
+  const std::vector<FillRect> rects = cut_rects(whole);
   p.n = (int)rects.size();
   if (!p.n) return NYX_OK;
   std::vector<long long> pref(p.n);
