@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(FusedGeom<R, TX, TY>::NT, 1) k_fused(nyx::Fuse
 // Coefficient 1 - max_d flat_d of every cell of [-1, n]^3 of every box (the
 // cells the advance traces; the +-3 stencil fits in the 4 ghost cells), from
 // the primitives exactly as the advance forms them in type R.  One block per
-// tile of output columns (nyx::FlatTile) walks the planes c = -1 .. n_z: it
+// tile of output columns (nyx::FlatTile) walks its planes c: it
 // keeps p and u_z of planes c-3 .. c+3 at the output columns in a ring, and
 // p, u_x, u_y of plane c on the tile's frame (+-3 in x and y), so that each
 // cell's primitives are formed about once per tile instead of once per
@@ -770,7 +770,10 @@ __global__ void __launch_bounds__(FusedGeom<R, TX, TY>::NT, 1) k_fused(nyx::Fuse
 constexpr int FLAT_TX = 34, FLAT_TY = 17;  // largest output tile
 constexpr int FLAT_NO = FLAT_TX * FLAT_TY;
 constexpr int FLAT_NF = (FLAT_TX + 6) * (FLAT_TY + 6);
-constexpr int FLAT_THREADS = 512;
+// Five blocks fit an SM in FP32 (43.4 KB of shared memory each) at 320 threads
+// of 40 registers: the planes of one block load while others compute (one
+// 192^3 box: 257 us; 385 us with 512 threads, which fitted twice).
+constexpr int FLAT_THREADS = 320;
 
 template <class R>
 constexpr size_t flat_smem() {
@@ -780,10 +783,9 @@ constexpr size_t flat_smem() {
 __device__ __forceinline__ int flat_slot(int k) { return (k + 7) % 7; }  // k >= -7
 
 template <class R>
-__global__ void __launch_bounds__(FLAT_THREADS) k_flatten(const nyx::BoxDev *boxes,
-                                                          const nyx::FlatTile *tiles,
-                                                          const double *Sall,
-                                                          const nyx::SchemeConsts *K, R *FLall) {
+__global__ void __launch_bounds__(FLAT_THREADS, sizeof(R) == 4 ? 5 : 2)
+    k_flatten(const nyx::BoxDev *boxes, const nyx::FlatTile *tiles, const double *Sall,
+              const nyx::SchemeConsts *K, R *FLall) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   R *ringp = reinterpret_cast<R *>(smem_raw);  // [7][FLAT_NO] p at the output columns
   R *ringw = ringp + 7 * FLAT_NO;               // [7][FLAT_NO] u_z at the output columns
@@ -810,8 +812,8 @@ __global__ void __launch_bounds__(FLAT_THREADS) k_flatten(const nyx::BoxDev *box
       U[o] = q[3];
     }
   };
-  for (int k = -4; k <= 1; ++k) ring_plane(k);
-  for (int c = -1; c <= b.n[2]; ++c) {
+  for (int k = T.z0 - 3; k < T.z0 + 3; ++k) ring_plane(k);
+  for (int c = T.z0; c < T.z0 + T.nz; ++c) {
     ring_plane(c + 3);
     for (int e = threadIdx.x; e < NF; e += blockDim.x) {
       R q[5];

@@ -60,14 +60,14 @@ struct FillRect {
   int dlo[3], ext[3], slo[3], sstep[3];
 };
 
-// Work item of the fused persistent kernel: a TX x TY column tile of a box.
-// Output tile of the shock-flattening pass: columns [x0, x0+nx) x [y0, y0+ny)
-// of one box, local coordinates (-1 and n are the one-cell halo); nx <= 34,
-// ny <= 17.
+// Output tile of the shock-flattening pass: columns [x0, x0+nx) x [y0, y0+ny),
+// planes [z0, z0+nz) of one box, local coordinates (-1 and n are the one-cell
+// halo); nx <= 34, ny <= 17.
 struct FlatTile {
-  int box, x0, y0, nx, ny;
+  int box, x0, y0, nx, ny, z0, nz;
 };
 
+// Work item of the fused persistent kernel: a TX x TY column tile of a box.
 struct WorkItem {
   int box;
   int x0, y0;
