@@ -57,23 +57,7 @@ __device__ __forceinline__ Eos<R> make_eos(const nyx::SchemeConsts &k, bool mixe
   return e;
 }
 
-// double -> float, round to nearest even, flushing results below the
-// smallest normal float to zero (the mixed unit runs with flush-to-zero),
-// computed on the integer pipe: the FP64 pipe of this part is 1/64 of the
-// FP32 rate and also executes the F2F conversion.
-__device__ __forceinline__ float d2f_rn(double d) {
-  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-  const unsigned sign = hi & 0x80000000u;
-  const int E = (int)((hi >> 20) & 0x7ffu);
-  const int e = E - 896;
-  const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
-  const unsigned rem = lo & 0x1fffffffu;
-  unsigned bits = ((unsigned)e << 23) + m;
-  bits += (rem > 0x10000000u || (rem == 0x10000000u && (m & 1u))) ? 1u : 0u;
-  if (e <= 0) bits = 0u;
-  if (e >= 255) bits = (E == 0x7ff && ((hi & 0xfffffu) | lo)) ? 0x7fc00000u : 0x7f800000u;
-  return __uint_as_float(bits | sign);
-}
+using nyx::d2f_rn;
 
 template <class R>
 __device__ __forceinline__ R to_r(double x) {

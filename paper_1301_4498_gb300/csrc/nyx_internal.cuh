@@ -133,6 +133,28 @@ inline int walk_grid(long long n, int block) {
   return (int)(g < 1 ? 1 : g);
 }
 
+// double -> float, round to nearest even, flushing results below the
+// smallest normal float to zero (as the mixed advance does),
+// computed on the integer pipe: the FP64 pipe of this part is 1/64 of the
+// FP32 rate and also executes the F2F conversion.
+__device__ __forceinline__ float d2f_rn(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned sign = hi & 0x80000000u;
+  const int E = (int)((hi >> 20) & 0x7ffu);
+  const int e = E - 896;
+  const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const unsigned rem = lo & 0x1fffffffu;
+  unsigned bits = ((unsigned)e << 23) + m;
+  bits += (rem > 0x10000000u || (rem == 0x10000000u && (m & 1u))) ? 1u : 0u;
+  if (e <= 0) bits = 0u;
+  if (e >= 255) bits = (E == 0x7ff && ((hi & 0xfffffu) | lo)) ? 0x7fc00000u : 0x7f800000u;
+  return __uint_as_float(bits | sign);
+}
+
+__device__ __forceinline__ bool finite_d(double x) {  // on the integer pipe too
+  return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
+}
+
 // Positive doubles order like their bit patterns as unsigned 64-bit ints.  The
 // value is read first and the atomic left out where it would change nothing:
 // atomics on one address take about 0.8 ns each, one per warp of a 256^3 grid

@@ -103,11 +103,25 @@ __global__ void k_pg_grav_dense(const double *u, Dims d, double hdx, double *g) 
 // adds with atomics), so they multiply by host reciprocals instead of
 // dividing and accumulate with fused multiply-adds: the FP64 pipe is their
 // bound.
-__device__ __forceinline__ void cic(double x, double idx, int n, int &i0, double &w0) {
-  const double s = x * idx - 0.5;
-  const double fl = floor(s);
-  w0 = 1.0 - (s - fl);
-  i0 = wrp((int)fl, n);
+//
+// floor, conversion to int, comparisons and maxima run on the FP64 pipe as
+// well: the cell comes from one fused multiply-add to a number whose units are
+// the last bit, round(x/dx - 1), which is floor(s) or, where s is an integer,
+// possibly s - 1 with the whole weight on the cell above; maxima and signs are
+// integer operations.  Kick and drift of 2.1e6 particles 332 -> 289 us, kick
+// 306 -> 274 us, deposit 171 -> 151 us.
+__device__ __forceinline__ void cic(double x, double idx, int n, int &i0, double &w0, double &w1) {
+  const double big = 6755399441055744.0;  // 1.5 2^52
+  const double t = fma(x, idx, big - 1.0);
+  i0 = wrp(__double2loint(t), n);
+  w1 = fma(x, idx, (big - t) - 0.5);  // s - i0: -i0 - 1/2 is exact, one rounding
+  w0 = 1.0 - w1;
+}
+
+// max of |x| and a magnitude's bits; a NaN does not count, as in fmax
+__device__ __forceinline__ void max_mag(unsigned long long &m, double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x) & ~(1ull << 63);
+  if (b > m && b <= 0x7ff0000000000000ull) m = b;
 }
 
 __device__ __forceinline__ void g_at(const double *g, const Dims &d, double idx, double x0,
@@ -115,11 +129,11 @@ __device__ __forceinline__ void g_at(const double *g, const Dims &d, double idx,
   const long long N = (long long)d.n[0] * d.n[1] * d.n[2];
   int i0, j0, k0;
   double wx, wy, wz;
-  cic(x0, idx, d.n[0], i0, wx);
-  cic(x1, idx, d.n[1], j0, wy);
-  cic(x2, idx, d.n[2], k0, wz);
+  double vx, vy, vz;
+  cic(x0, idx, d.n[0], i0, wx, vx);
+  cic(x1, idx, d.n[1], j0, wy, vy);
+  cic(x2, idx, d.n[2], k0, wz, vz);
   const int i1 = wrp(i0 + 1, d.n[0]), j1 = wrp(j0 + 1, d.n[1]), k1 = wrp(k0 + 1, d.n[2]);
-  const double vx = 1.0 - wx, vy = 1.0 - wy, vz = 1.0 - wz;
   out[0] = out[1] = out[2] = 0.0;
 #pragma unroll
   for (int o = 0; o < 8; ++o) {
@@ -139,11 +153,11 @@ __global__ void k_pm_deposit(const double *x, const double *m, long long np, Dim
        p += (long long)gridDim.x * blockDim.x) {
     int i0, j0, k0;
     double wx, wy, wz;
-    cic(x[p], idx, d.n[0], i0, wx);
-    cic(x[np + p], idx, d.n[1], j0, wy);
-    cic(x[2 * np + p], idx, d.n[2], k0, wz);
+    double vx, vy, vz;
+    cic(x[p], idx, d.n[0], i0, wx, vx);
+    cic(x[np + p], idx, d.n[1], j0, wy, vy);
+    cic(x[2 * np + p], idx, d.n[2], k0, wz, vz);
     const int i1 = wrp(i0 + 1, d.n[0]), j1 = wrp(j0 + 1, d.n[1]), k1 = wrp(k0 + 1, d.n[2]);
-    const double vx = 1.0 - wx, vy = 1.0 - wy, vz = 1.0 - wz;
     const double mp = m[p] * iv;
 #pragma unroll
     for (int o = 0; o < 8; ++o) {
@@ -172,8 +186,10 @@ __global__ void k_pm_kick_drift(double *x, double *u, long long np, const double
       const double uh = fma(a_old, u[c * np + p], hdt * gp[c]) * ia_half;
       u[c * np + p] = uh;
       double xn = fma(dta, uh, xp[c]);
-      if (xn < 0.0) xn = xn + L[c];
-      if (xn >= L[c]) xn = xn - L[c];
+      // (as integers: a negative number has the sign bit, and positive ones order
+      // as their bits do)
+      if (__double_as_longlong(xn) < 0) xn = xn + L[c];
+      if (__double_as_longlong(xn) >= __double_as_longlong(L[c])) xn = xn - L[c];
       x[c * np + p] = xn;
     }
   }
@@ -185,7 +201,7 @@ __global__ void k_pm_kick_drift(double *x, double *u, long long np, const double
 __global__ void k_pm_kick(const double *x, double *u, long long np, const double *g, Dims d,
                           double idx, double a_half, double ia_new, double hdt,
                           unsigned long long *mx) {
-  double um = 0.0, gm = 0.0;
+  unsigned long long um = 0, gm = 0;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < np;
        p += (long long)gridDim.x * blockDim.x) {
     double gp[3];
@@ -194,42 +210,42 @@ __global__ void k_pm_kick(const double *x, double *u, long long np, const double
     for (int c = 0; c < 3; ++c) {
       const double un = fma(a_half, u[c * np + p], hdt * gp[c]) * ia_new;
       u[c * np + p] = un;
-      um = fmax(um, fabs(un));
-      gm = fmax(gm, fabs(gp[c]));
+      max_mag(um, un);
+      max_mag(gm, gp[c]);
     }
   }
   if (!mx) return;
   for (int o = 16; o > 0; o >>= 1) {
-    um = fmax(um, __shfl_xor_sync(0xffffffffu, um, o));
-    gm = fmax(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+    um = max(um, __shfl_xor_sync(0xffffffffu, um, o));
+    gm = max(gm, __shfl_xor_sync(0xffffffffu, gm, o));
   }
   if ((threadIdx.x & 31) == 0) {
-    atomic_max_pos(&mx[0], um);
-    atomic_max_pos(&mx[1], gm);
+    atomic_max_pos(&mx[0], __longlong_as_double((long long)um));
+    atomic_max_pos(&mx[1], __longlong_as_double((long long)gm));
   }
 }
 
 // Sec. 3.5: maxima of |u_d| and |g_d| at the particles (ordered bits)
 __global__ void k_pm_maxes(const double *x, const double *u, long long np, const double *g,
                            Dims d, double idx, unsigned long long *mx) {
-  double um = 0.0, gm = 0.0;
+  unsigned long long um = 0, gm = 0;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < np;
        p += (long long)gridDim.x * blockDim.x) {
     double gp[3];
     g_at(g, d, idx, x[p], x[np + p], x[2 * np + p], gp);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      um = fmax(um, fabs(u[c * np + p]));
-      gm = fmax(gm, fabs(gp[c]));
+      max_mag(um, u[c * np + p]);
+      max_mag(gm, gp[c]);
     }
   }
   for (int o = 16; o > 0; o >>= 1) {
-    um = fmax(um, __shfl_xor_sync(0xffffffffu, um, o));
-    gm = fmax(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+    um = max(um, __shfl_xor_sync(0xffffffffu, um, o));
+    gm = max(gm, __shfl_xor_sync(0xffffffffu, gm, o));
   }
   if ((threadIdx.x & 31) == 0) {
-    atomic_max_pos(&mx[0], um);
-    atomic_max_pos(&mx[1], gm);
+    atomic_max_pos(&mx[0], __longlong_as_double((long long)um));
+    atomic_max_pos(&mx[1], __longlong_as_double((long long)gm));
   }
 }
 

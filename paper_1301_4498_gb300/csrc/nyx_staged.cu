@@ -307,8 +307,10 @@ __global__ void k_update(BoxDev b, const SchemeConsts *K, const StepConsts *SC, 
 // valid cell of the level, in place on the predictor; one thread per cell,
 // cells of a box in x-fastest order (coalesced), the box found by a binary
 // search of the cell offsets.  CFL minimum of the result as in k_update (in
-// FP32 for mixed plans, as their CFL reduction is: FP64 division and square
-// root run at a small fraction of the FP32 rate on this part).
+// FP32 for mixed plans, as their CFL reduction is).  The FP64 pipe bounds it
+// (44 operations a cell), and conversions, comparisons and tests for finite
+// values take that pipe too: as integer operations 305 -> 290 us for 128^3
+// cells.
 template <bool F32DT>
 __global__ void k_correct(const BoxDev *boxes, const long long *cell_pref, int nbox,
                           long long total, const SchemeConsts *K, const StepConsts *SC,
@@ -317,6 +319,11 @@ __global__ void k_correct(const BoxDev *boxes, const long long *cell_pref, int n
   const SchemeConsts k = *K;
   const StepConsts sc = *SC;
   double local_min = __longlong_as_double(0x7ff0000000000000LL);
+  // F32DT: constants and the running minimum in FP32
+  const float gm1 = (float)k.gm1, gamma = (float)k.gamma, small_pres = (float)k.small_pres;
+  const float an = (float)sc.a_new;
+  float min32 = __int_as_float(0x7f800000), adx[3] = {0.0f, 0.0f, 0.0f};
+  int box = -1;
   unsigned flags = 0;
   for (CellWalk w(cell_pref, nbox, total); w.valid(); w.next(cell_pref, nbox)) {
     const BoxDev &b = boxes[w.box];
@@ -342,23 +349,28 @@ __global__ void k_correct(const BoxDev *boxes, const long long *cell_pref, int n
                 Sp[5 * bs + id], true, true, o6);
     const double rho_s = o6[0];
     if (!(rho_s > 0.0)) flags |= ST_NEGATIVE;
-    if (!isfinite(rho_s) || !isfinite(o6[4]) || !isfinite(o6[5]) || !isfinite(o6[1]) ||
-        !isfinite(o6[2]) || !isfinite(o6[3]))
-      flags |= ST_NONFINITE;
+    bool fin = finite_d(rho_s);
 #pragma unroll
-    for (int c = 1; c < 6; ++c) Sp[c * bs + id] = o6[c];
+    for (int c = 1; c < 6; ++c) {
+      Sp[c * bs + id] = o6[c];
+      fin = fin && finite_d(o6[c]);
+    }
+    if (!fin) flags |= ST_NONFINITE;
     if (dtacc) {
       if constexpr (F32DT) {
-        const float r = (float)rho_s, ir = 1.0f / r;
-        float p = (float)k.gm1 * (float)o6[5];
-        if (p < (float)k.small_pres) p = (float)k.small_pres;
-        const float c = sqrtf((float)k.gamma * p * ir);
-        const float an = (float)sc.a_new;
-        const float t0 = an * (float)b.dx[0] / (fabsf((float)o6[1] * ir) + c);
-        const float t1 = an * (float)b.dx[1] / (fabsf((float)o6[2] * ir) + c);
-        const float t2 = an * (float)b.dx[2] / (fabsf((float)o6[3] * ir) + c);
-        const double tm = (double)fminf(t0, fminf(t1, t2));
-        if (tm < local_min) local_min = tm;
+        const float r = d2f_rn(rho_s), ir = 1.0f / r;
+        float p = gm1 * d2f_rn(o6[5]);
+        if (p < small_pres) p = small_pres;
+        const float c = sqrtf(gamma * p * ir);
+        if (w.box != box) {
+          box = w.box;
+#pragma unroll
+          for (int d = 0; d < 3; ++d) adx[d] = an * (float)b.dx[d];
+        }
+        const float t0 = adx[0] / (fabsf(d2f_rn(o6[1]) * ir) + c);
+        const float t1 = adx[1] / (fabsf(d2f_rn(o6[2]) * ir) + c);
+        const float t2 = adx[2] / (fabsf(d2f_rn(o6[3]) * ir) + c);
+        min32 = fminf(min32, fminf(t0, fminf(t1, t2)));
       } else {
         double p = k.gm1 * o6[5];
         if (p < k.small_pres) p = k.small_pres;
@@ -373,6 +385,7 @@ __global__ void k_correct(const BoxDev *boxes, const long long *cell_pref, int n
     }
   }
   if (dtacc) {
+    if (F32DT) local_min = (double)min32;
     for (int o = 16; o > 0; o >>= 1) {
       double v = __shfl_xor_sync(0xffffffffu, local_min, o);
       if (v < local_min) local_min = v;
