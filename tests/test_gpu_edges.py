@@ -1,0 +1,192 @@
+"""The splits of the work at the sizes where they can go wrong: columns cut
+down to single planes, ghost rectangles and flattening columns cut into
+pieces, scheme variants with their own instantiation, non-finite fluxes, and
+the mixed Poisson solve on grids that its tiles do not divide, with other
+sweep counts, from a given potential and at scales that fixed point cannot
+hold."""
+import itertools
+
+import numpy as np
+import pytest
+
+import oracle
+from gates import MIXED_GATES
+from paper_1301_4498_gb300 import workloads as W
+
+import test_oracle_amr as TA
+
+pytestmark = pytest.mark.gpu
+H = pytest.importorskip("paper_1301_4498_gb300.hydro")
+torch = pytest.importorskip("torch")
+
+
+def _boxes(extents, sigma=0.5, seed=11, bc=None):
+    """Independent comoving boxes (or one box with boundary types bc)."""
+    lev = (W.single_box_level(*extents[0], 1.0 / 64, bc) if bc
+           else W.independent_boxes_level(extents, 1.0 / 64))
+    S, G = [], []
+    for b, (nx, ny, nz) in enumerate(extents):
+        s, g = W._patch_state(lev, b, W.comoving_fields((nz, ny, nx), sigma, seed + b, 1.0 / 64))
+        S.append(s)
+        G.append(g)
+    return lev, S, G
+
+
+def _step(lev, S, G, dt, **kw):
+    """One step of a given dt: the plan and the new state per box."""
+    plan = H.Plan(lev, gamma=5.0 / 3.0, cfl=0.5, **kw)
+    L = H.make_level(plan, S, G)
+    a = torch.tensor([0.02, 0.0201], dtype=torch.float64, device="cuda")
+    d = torch.tensor([dt, 0.0], dtype=torch.float64, device="cuda")
+    plan.run(L, a, d, 1, compute_dt0=False, use_graph=False)
+    torch.cuda.synchronize()
+    return plan, plan.from_device(L.current, 6)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("extent", [(4, 4, 4), (8, 8, 6), (18, 10, 16), (34, 6, 30)])
+def test_cut_columns_give_the_bits_of_whole_ones(extent, precision):
+    # alone, the box's columns are cut until every SM has an item; among 1000
+    # others they stay whole: the same cells from the same operations
+    fill = [(16, 8, 4)] * 1000
+    lev, S, G = _boxes([extent])
+    p1, one = _step(lev, S, G, 1e-5, precision=precision)
+    s0, g0 = S[0], G[0]
+    lev2 = W.independent_boxes_level([extent] + fill, 1.0 / 64)
+    f = W.comoving_fields((4, 8, 16), 0.5, 3, 1.0 / 64)
+    s1, g1 = W._patch_state(lev2, 1, f)
+    p2, many = _step(lev2, [s0] + [s1] * len(fill), [g0] + [g1] * len(fill), 1e-5,
+                     precision=precision)
+    assert p1.status() == (0, 0) and p2.status() == (0, 0)
+    assert np.array_equal(W.valid(one[0]), W.valid(many[0]))
+    p1.close()
+    p2.close()
+
+
+@pytest.mark.parametrize("bc", [(0,) * 6, (1,) * 6, (1, 0, 1, 1, 0, 1)])
+@pytest.mark.parametrize("extent", [(4, 6, 8), (6, 130, 38), (130, 34, 6), (64, 64, 64)])
+def test_cut_ghost_rectangles(extent, bc):
+    lev, S, _ = _boxes([extent], bc=bc)
+    plan = H.Plan(lev, gamma=1.4, cfl=0.5)
+    for ncomp in (6, 3, 2):
+        ref = [S[0][:ncomp].copy()]
+        dev = plan.to_device(ref, ncomp)
+        plan.fill(dev, ncomp)
+        torch.cuda.synchronize()
+        got = plan.from_device(dev, ncomp)
+        oracle.fill_ghosts(lev, ref)
+        assert np.array_equal(got[0], ref[0])
+    plan.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("extent", [(4, 4, 4), (32, 14, 6), (34, 16, 10), (70, 36, 30)])
+def test_cut_flattening_columns(extent, precision):
+    lev, S, G = _boxes([extent], sigma=1.0)
+    P = oracle.OracleParams(gamma=5.0 / 3.0, cfl=0.5, flattening=1)
+    plan, got = _step(lev, S, G, 1e-5, precision=precision, flattening=True)
+    assert plan.status() == (0, 0)
+    ref = oracle.advance(lev, P, S, G, a_old=0.02, a_new=0.0201, dt=1e-5)[0]
+    tol = 1e-12 if precision == "fp64" else MIXED_GATES["linf"]
+    for c in range(6):
+        g, r = W.valid(got[0])[c], W.valid(ref[0])[c]
+        assert np.abs(g - r).max() <= tol * np.abs(r).max()
+    plan.close()
+
+
+@pytest.mark.parametrize("plm,linear,flat", list(itertools.product((0, 1), repeat=3)))
+def test_variants_of_the_mixed_default_shape(plm, linear, flat):
+    lev, S, G = _boxes([(18, 10, 14)], sigma=0.7)
+    kw = dict(grav_energy=1, reconstruction=plm, riemann_solver=linear)
+    P = oracle.OracleParams(gamma=5.0 / 3.0, cfl=0.5, flattening=flat, **kw)
+    plan, got = _step(lev, S, G, 1e-5, precision="mixed", flattening=bool(flat), grav_energy=1,
+                      reconstruction="plm" if plm else "ppm",
+                      riemann_solver="linear" if linear else "two_shock")
+    assert plan.status() == (0, 0) and plan.tile_shape()[0] == 3
+    ref = oracle.advance(lev, P, S, G, a_old=0.02, a_new=0.0201, dt=1e-5)[0]
+    for c in range(6):
+        g, r = W.valid(got[0])[c], W.valid(ref[0])[c]
+        assert np.abs(g - r).max() <= MIXED_GATES["linf"] * np.abs(r).max()
+    plan.close()
+
+
+@pytest.mark.parametrize("comp,value", [(0, np.nan), (1, np.nan), (1, np.inf), (2, -np.inf),
+                                        (5, np.nan), (5, np.inf)])
+@pytest.mark.parametrize("where", [(0, 0, 0), (17, 9, 13), (9, 7, 6)])
+def test_non_finite_cells_reach_the_status(where, comp, value):
+    lev, S, G = _boxes([(18, 10, 14)])
+    i, j, k = where
+    W.valid(S[0])[comp, k, j, i] = value
+    plan, _ = _step(lev, S, G, 1e-5, precision="mixed")
+    rc, flags = plan.status()
+    assert rc != 0 and flags != 0
+    plan.close()
+
+
+def test_interpolation_ignores_nan_neighbours_as_the_oracle_does():
+    w, fine = TA._hierarchy()
+    cp = H.Plan(w.level, precision="fp64", keep_fluxes=1)
+    fp = H.Plan(fine, stream=cp.torch_stream, precision="fp64", keep_fluxes=1, coarse_fine=1)
+    amr = H.Amr(cp, fp)
+    cs = TA._filled(w.level, w.state)
+    rng = np.random.default_rng(4)
+    for s in cs:
+        for c in range(6):
+            for z, y, x in rng.integers(0, s.shape[1], (40, 3)):
+                s[c, z, y, x] = np.nan
+    ref = oracle.amr_interp(w.level, cs, fine, TA._fine_empty(fine, 6), "all")
+    dev = fp.empty_field(6)
+    amr.interp(cp.to_device(cs, 6), dev, 6, "all")
+    torch.cuda.synchronize()
+    for g, r in zip(fp.from_device(dev, 6), ref):
+        assert np.array_equal(g, r, equal_nan=True)
+    amr.close(); fp.close(); cp.close()
+
+
+def _spectral_phi(f, h):
+    """Zero-mean solution of the 7-point Laplacian: the operator is diagonal in
+    Fourier space."""
+    F = np.fft.fftn(f)
+    lam = 0.0
+    for ax, n in enumerate(f.shape):
+        s = [1, 1, 1]
+        s[ax] = n
+        lam = lam - (4.0 / h**2) * (np.sin(np.pi * np.arange(n) / n)**2).reshape(s)
+    lam = np.broadcast_to(lam, f.shape).copy()
+    lam[0, 0, 0] = 1.0
+    F /= lam
+    F[0, 0, 0] = 0.0
+    return np.fft.ifftn(F).real
+
+
+@pytest.mark.parametrize("n,prm,scale,warm", [
+    (8, {}, 1.0, False), (20, {}, 1.0, False), (36, {}, 1.0, True), (64, {}, 1.0, False),
+    (100, {}, 1.0, False), (128, {}, 1.0, True),
+    (48, dict(pre=1, post=1), 1.0, False), (48, dict(pre=3, post=2), 1.0, True),
+    (48, dict(pre=0, post=3), 1.0, False), (48, dict(pre=2, post=0), 1.0, True),
+    (32, {}, 1e-14, False), (32, {}, 1e12, True), (32, {}, 1e-30, False), (32, {}, 1e25, True)])
+def test_mixed_poisson_solve(n, prm, scale, warm):
+    lev = W.single_box_level(n, n, n, 1.0 / n)
+    rng = np.random.default_rng(n)
+    arr = np.zeros(lev.shape(0, 6))
+    W.valid(arr)[0] = np.exp(rng.standard_normal((n, n, n)))
+    plan = H.Plan(lev, precision="fp64")
+    L = H.make_level(plan, [arr], None)
+    tol = 1e-11
+    ps = H.Poisson(plan, four_pi_G=scale, precision="mixed", tol=tol, max_cycles=200, **prm)
+    if warm:  # from the potential of another density
+        other = np.zeros_like(arr)
+        W.valid(other)[0] = 1.0 + rng.random((n, n, n))
+        ps.solve(plan.to_device([other], 6), 0.5, None, warm_start=False)
+    cyc, res = ps.solve(L.current, 0.5, None, warm_start=warm)
+    phi = ps.phi().cpu().numpy()
+    rho = W.valid(arr)[0]
+    f = scale / 0.5 * (rho - rho.mean())
+    ref = _spectral_phi(f, 1.0 / n)
+    phi = phi - phi.mean()
+    # a residual of max norm r leaves an error of at most 0.26 l^2 r (the zero-mean
+    # inverse of the operator on a periodic box of side l = 1)
+    assert 0 < cyc and res <= tol
+    assert np.abs(phi - ref).max() <= 0.26 * tol * np.abs(f).max() + 1e-12 * np.abs(ref).max()
+    ps.close()
+    plan.close()
