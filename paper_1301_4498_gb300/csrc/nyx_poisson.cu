@@ -689,12 +689,14 @@ __global__ void __launch_bounds__(kTailThreads) k_pg_tail(const TailArgs<T> a) {
 // one colour and their neighbours (all of the other colour) lie at consecutive
 // addresses, free of bank conflicts.
 //
-// Bound: shared memory (9 accesses per relaxed cell; memory would allow 30 us
-// for the 12 B per cell of a sweep).  A sweep of a 256^3 grid: 114 us with the
-// colours split (74 us from zero), 120 us with even and odd x split (two-way conflicts), against
-// 2 x 37 us per half-sweep launch plus the transfers' own passes.
+// Bound: issue and barriers (60 % of issue slots at three CTAs per SM; memory
+// would allow 30 us for the 12 B per cell of a sweep).  A sweep of a 256^3 grid:
+// 110 us (71 us from zero) with the colours split and two cells of a colour per
+// access, 120 us with even and odd x split (two-way conflicts), against 2 x 37 us
+// per half-sweep launch plus the transfers' own passes.  288 threads: the 792
+// pairs of a plane in three rounds (four of 256 threads took 3 % longer).
 constexpr int kSwTX = 64, kSwTY = 16, kSwH = 36, kSwW = 2 * kSwH, kSwR = kSwTY + 6;
-constexpr int kSwThreads = 256, kSwPlane = kSwW * kSwR, kSwPairs = kSwH * kSwR;
+constexpr int kSwThreads = 288, kSwPlane = kSwW * kSwR, kSwPairs = kSwH * kSwR;
 constexpr int kSwC = kSwPairs;  // offset of the black cells of a plane
 constexpr int kSwLoads = (kSwPairs + kSwThreads - 1) / kSwThreads;
 constexpr size_t kSwSmem = sizeof(float) * 11 * kSwPlane;
@@ -765,17 +767,19 @@ __global__ void __launch_bounds__(kSwThreads, 3) k_pg_smooth(const float *phi_in
   };
   auto plane = [&](int t) { return sp + (t + 6 * 8) % 6 * kSwPlane; };
   auto fplane = [&](int t) { return sf + (t + 5 * 8) % 5 * kSwPlane; };
-  // this thread's cells to relax, 36 a row (the outermost only get values that
-  // nothing uses): red ones of rows 1 .. kSwR - 2, black ones of rows 2 .. kSwR - 3
-  constexpr int kRelax = (kSwR - 2) * kSwH;
+  // cells to relax, two of a colour at a time, 18 pairs a row (the outermost only
+  // get values that nothing uses): red ones of rows 1 .. kSwR - 2, black ones of
+  // rows 2 .. kSwR - 3
+  constexpr int kRelax = (kSwR - 2) * kSwH / 2;
   constexpr int kIter = (kRelax + kSwThreads - 1) / kSwThreads;
   unsigned odd = 0, inner = 0;
 #pragma unroll
   for (int u = 0; u < kIter; ++u) {
-    const int row = 1 + (tid + u * kSwThreads) / kSwH;
+    const int row = 1 + 2 * (tid + u * kSwThreads) / kSwH;
     odd |= (unsigned)((y0 + row - 3) & 1) << u;
     inner |= (unsigned)(row >= 2 && row <= kSwR - 3) << u;
   }
+  auto two = [](const float *p) { return *reinterpret_cast<const float2 *>(p); };
   auto relax = [&](int t, int color) {
     float *P = plane(t) + color * kSwC;
     const int oc = (1 - color) * kSwC;
@@ -783,10 +787,19 @@ __global__ void __launch_bounds__(kSwThreads, 3) k_pg_smooth(const float *phi_in
     const float *F = fplane(t) + color * kSwC;
 #pragma unroll
     for (int u = 0; u < kIter; ++u) {
-      const int e = tid + u * kSwThreads, a = kSwH + e;
+      const int e = tid + u * kSwThreads, a = kSwH + 2 * e;
       if (e >= kRelax || (color && !((inner >> u) & 1u))) continue;
       const int px = (int)((odd >> u) ^ (unsigned)(t + color)) & 1;
-      P[a] = (nb(Q, Pm, Pp, a, px) - h2 * F[a]) * (1.0f / 6.0f);
+      const float2 q = two(Q + a), ym = two(Q + a - kSwH), yp = two(Q + a + kSwH);
+      const float2 zm = two(Pm + a), zp = two(Pp + a), ff = two(F + a);
+      const float o = Q[px ? a + 2 : a - 1];
+      // left + right: (o, q.x) + q for even x, q + (q.y, o) for odd x
+      float2 v = px ? make_float2(q.x + q.y, q.y + o) : make_float2(o + q.x, q.x + q.y);
+      v.x = (((v.x + ym.x) + yp.x) + zm.x) + zp.x;
+      v.y = (((v.y + ym.y) + yp.y) + zm.y) + zp.y;
+      v.x = (v.x - h2 * ff.x) * (1.0f / 6.0f);
+      v.y = (v.y - h2 * ff.y) * (1.0f / 6.0f);
+      *reinterpret_cast<float2 *>(P + a) = v;
     }
   };
   float racc = 0.0f;  // this thread's coarse cell: residuals summed so far
@@ -811,9 +824,9 @@ __global__ void __launch_bounds__(kSwThreads, 3) k_pg_smooth(const float *phi_in
       if (t + 2 <= z1 + 2) load(t + 2, R);
     }
     __syncthreads();
-    if (RESTRICT && t - 4 >= z0 && t - 4 < z1) {
+    const int I = tid & 31, J = tid >> 5;  // coarse cell of the tile (J < kSwTY / 2)
+    if (RESTRICT && t - 4 >= z0 && t - 4 < z1 && J < kSwTY / 2) {
       const int q = t - 4;
-      const int I = tid & 31, J = tid >> 5;
 #pragma unroll
       for (int o = 0; o < 4; ++o) {
         const int px = o & 1, row = 3 + 2 * J + (o >> 1), a = row * kSwH + 2 + I;
@@ -1057,15 +1070,32 @@ void vcycle(nyx_poisson *S, std::vector<LevelT<T>> &L, size_t l, size_t tail_at,
 }
 
 // One fused sweep of FP32 grid l from phi_in into phi_out.
+// Planes per CTA of the fused sweeps: even (a coarse plane stays in one CTA).  A
+// CTA takes 7 steps more than planes, and a step about 1 us alone on an SM, 1.42
+// and 1.85 us with one or two others (three fit; 128^3 grid); of the even
+// numbers of planes the one with the shortest sum.
+int smooth_planes(int tiles, int nz) {
+  static const double step[4] = {0.0, 0.99, 1.42, 1.85};
+  int best = 2;
+  double least = 1e300;
+  for (int zc = 2; zc - 1 <= nz; zc += 2) {
+    const long long ctas = (long long)tiles * ((nz + zc - 1) / zc);
+    const long long full = ctas / (3 * 152), left = (ctas % (3 * 152) + 151) / 152;
+    const double t = (zc + 7) * (full * step[3] + step[left]);
+    if (t < least) {
+      least = t;
+      best = zc;
+    }
+  }
+  return best;
+}
+
 template <bool ZERO, bool PROLONG, bool RESTRICT, int ADD>
 void smooth_launch(nyx_poisson *S, size_t l, const float *in, float *out, const float *pc) {
   const LevelT<float> &g = S->L32[l];
   const LevelT<float> &c = S->L32[std::min(l + 1, S->L32.size() - 1)];
   const int tx = (g.d.n[0] + kSwTX - 1) / kSwTX, ty = (g.d.n[1] + kSwTY - 1) / kSwTY;
-  // planes per CTA: even (a coarse plane stays in one CTA), and as many CTAs as
-  // are resident at once (three per SM by shared memory)
-  const int nch = std::max(1, 3 * 152 / (tx * ty));
-  const int zc = std::max(2, ((g.d.n[2] + nch - 1) / nch + 1) & ~1);
+  const int zc = smooth_planes(tx * ty, g.d.n[2]);
   const dim3 grid(tx, ty, (g.d.n[2] + zc - 1) / zc);
   k_pg_smooth<ZERO, PROLONG, RESTRICT, ADD><<<grid, kSwThreads, kSwSmem, S->P->stream>>>(
       in, g.f, out, g.d, g.h2, g.ih2, zc, pc, c.f, c.d, S->L[0].phi, S->d_fix, S->fix_s);
