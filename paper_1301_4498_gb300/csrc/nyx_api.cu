@@ -735,19 +735,31 @@ int part_groups(nyx_plan::RunPart &pt, const std::vector<int> &gb) {
 // long as each group keeps 2 waves of items or more in the plan's tile shape
 // (4 waves of the task form's half-size items for a run on the device, where a
 // group's tail costs more than its overlapped fill gains: 563 boxes, two
-// steps, 32.0 ms with 9 groups, 32.1 ms with 18).  One group (no overlap)
+// steps, 32.0 ms with 9 groups, 32.1 ms with 18; a run takes groups that a host
+// step made only where its own rule gives two or more).  One group (no overlap)
 // otherwise.  Every shape gets the same groups.  (On the 512^3 large level:
 // 32 groups 1.74e9 zone-updates/s end to end, 16 groups 1.72e9, 8 groups
 // 1.59e9.)
 int setup_readback(nyx_plan *P, bool host) {
   const int nsh = fused_num_shapes(P->prm.precision);
-  int waves = P->nitems[P->shape] / std::max(1, P->max_grid[P->shape]);
+  const int grid = std::max(1, P->max_grid[P->shape]);
+  int waves = P->nitems[P->shape] / grid, begun = (P->nitems[P->shape] + grid - 1) / grid;
   if (!P->parts.empty()) {
-    waves = 0;
-    for (const auto &pt : P->parts) waves += pt.nitems / std::max(1, pt.grid);
+    waves = begun = 0;
+    for (const auto &pt : P->parts) {
+      const int pg = std::max(1, pt.grid);
+      waves += pt.nitems / pg;
+      begun += (pt.nitems + pg - 1) / pg;
+    }
   }
-  const int per = host ? 2 : (fused_shape(P->shape).task ? 4 : 2);
-  const int G = std::min(std::min(32, P->nbox), waves / per);
+  const int dev = fused_shape(P->shape).task ? 4 : 2, per = host ? 2 : dev;
+  P->run_groups = waves / dev > 1;
+  // up to four groups also where that leaves them about a wave each: the copies
+  // in and out are what is worth hiding there (27 boxes, two, three and four
+  // groups: of 64^3 6.52, 6.09 and 5.95 ms, of 48^3 3.01, 2.92 and 2.84 ms; of
+  // 32^3, 1.4 waves, one and two groups: 1.03 and 0.95 ms)
+  const int least = host ? std::min(4, begun) : 0;
+  const int G = std::min(std::min(32, P->nbox), std::max(waves / per, least));
   std::vector<int> gb(1, 0);
   for (int g = 1; g < G; ++g) {
     const long long want = P->total_cells * g / G;
@@ -1277,7 +1289,7 @@ int enqueue_run(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev, 
   // advance; profiled runs keep one fill and one advance launch per step so
   // that each is timed on its own
   if (P->prm.batching != NYX_PER_BOX && P->ngrp > 1 && !(P->prm.autotune && !P->tuned) &&
-      !P->profiling && nsteps > 0) {
+      !P->profiling && P->run_groups && nsteps > 0) {
     return run_grouped(P, L, a_dev, dt_dev, nsteps);
   }
   for (int s = 0; s < nsteps; ++s) {

@@ -78,6 +78,7 @@ struct nyx_plan {
   // queue order), one launch per group; a group's cells are gathered and
   // copied to the host on copy_stream while the next group advances
   int ngrp = 0;
+  bool run_groups = false;  // also used by runs on the device
   std::vector<int> grp_box;
   std::vector<int> grp_off[8];  // per shape: first item of each group, ngrp + 1 entries
   nyx::WorkItem *d_items_grp[8] = {nullptr};
