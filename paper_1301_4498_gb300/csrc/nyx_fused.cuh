@@ -203,16 +203,6 @@ __device__ __forceinline__ double f2d_exact(float f) {
   return __hiloint2double((int)hi, (int)(b << 29));
 }
 
-// The same for a finite float in five integer instructions: zero becomes
-// 2^-127, below the rounding of whatever it is subtracted from (FP32 values
-// here are zero or at least 2^-126).  Non-finite values are the caller's to
-// handle.
-__device__ __forceinline__ double f2d_finite(float f) {
-  const unsigned b = __float_as_uint(f);
-  const unsigned hi = ((b >> 3) & 0x0fffffffu) + 0x38000000u;
-  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
-}
-
 // finite test on the high word (integer pipe)
 __device__ __forceinline__ bool finite_hi(double x) {
   return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
@@ -225,14 +215,12 @@ __device__ __forceinline__ bool finite_hi(double x) {
 // formed in FP32, 1/rho is an FP32 reciprocal refined by one FP64 Newton step.
 // FP32 constants of the mixed update (converted once per work item).
 struct MixK {
-  double idx[3];  // 1/dx
   float idx0, idx1, idx2, gm1, gamma, small_pres, an_dx0, an_dx1, an_dx2;
 };
 
 __device__ __forceinline__ MixK make_mixk(const nyx::SchemeConsts &k, const nyx::StepConsts &sc,
                                           const nyx::BoxDev &b) {
   MixK m;
-  for (int d = 0; d < 3; ++d) m.idx[d] = b.idx[d];
   m.idx0 = d2f_rn(b.idx[0]);
   m.idx1 = d2f_rn(b.idx[1]);
   m.idx2 = d2f_rn(b.idx[2]);
@@ -245,72 +233,45 @@ __device__ __forceinline__ MixK make_mixk(const nyx::SchemeConsts &k, const nyx:
   return m;
 }
 
-// State (rho, m_x, m_y, m_z, rhoE, rhoe) and gravity of one cell, loaded ahead
-// of its update.
-struct CellIn {
-  double s[6], g[3];
-};
-__device__ __forceinline__ CellIn load_cell(const double *S, const double *G, long long bs,
-                                            long long id) {
-  CellIn c;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) c.s[k] = S[k * bs + id];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) c.g[k] = G ? G[k * bs + id] : 0.0;
-  return c;
-}
-
-// F(k, f): component k of (rho, m_x, m_y, m_z, rhoE, rhoe, u, p) of the cell's
-// final flux on face f = 0..5 (x low, x high, y low, ...), fetched where it is
-// used.  all_finite: no flux is infinite or NaN (the fast conversion's
-// condition).  genergy: the second form of the gravity energy source.
-template <class Flux>
 __device__ __forceinline__ void update_cell_mixed(
-    const nyx::SchemeConsts &k, const nyx::StepConsts &sc, long long bs, const MixK &mk,
-    const CellIn &in, double *Sn, long long id, Flux F, float &dtmin, unsigned &flags,
-    bool want_dt, bool full, bool all_finite, bool genergy) {
+    const nyx::SchemeConsts &k, const nyx::StepConsts &sc, const nyx::BoxDev &b, const MixK &mk,
+    const double *S, const double *G, double *Sn, long long id, const float (&Fxm)[8],
+    const float (&Fxp)[8], const float (&Fym)[8], const float (&Fyp)[8], const float (&Fzm)[8],
+    const float (&Fzp)[8], float &dtmin, unsigned &flags, bool want_dt, bool full) {
+  const long long bs = b.stride;
   double div[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
-    const double xl = f2d_finite(F(c, 0));
-    const double dx_ = f2d_finite(F(c, 1)) - xl;
-    const double dy_ = f2d_finite(F(c, 3)) - f2d_finite(F(c, 2));
-    const double dz_ = f2d_finite(F(c, 5)) - f2d_finite(F(c, 4));
-    div[c] = dx_ * mk.idx[0] + dy_ * mk.idx[1] + dz_ * mk.idx[2];
+    const double dx_ = f2d_exact(Fxp[c]) - f2d_exact(Fxm[c]);
+    const double dy_ = f2d_exact(Fyp[c]) - f2d_exact(Fym[c]);
+    const double dz_ = f2d_exact(Fzp[c]) - f2d_exact(Fzm[c]);
+    div[c] = dx_ * b.idx[0] + dy_ * b.idx[1] + dz_ * b.idx[2];
   }
-  const float pdivu_f = 0.5f * (F(7, 1) + F(7, 0)) * (F(6, 1) - F(6, 0)) * mk.idx0 +
-                        0.5f * (F(7, 3) + F(7, 2)) * (F(6, 3) - F(6, 2)) * mk.idx1 +
-                        0.5f * (F(7, 5) + F(7, 4)) * (F(6, 5) - F(6, 4)) * mk.idx2;
-  if (!all_finite) {  // rare: infinite or NaN fluxes make their divergence NaN
-#pragma unroll 1
-    for (int c = 0; c < 6; ++c) {
-      bool bad = false;
-#pragma unroll 1
-      for (int f = 0; f < 6; ++f) bad |= !(fabsf(F(c, f)) <= 3.402823466e38f);
-      if (bad) {
-#pragma unroll
-        for (int e = 0; e < 6; ++e)
-          if (e == c) div[e] = __longlong_as_double(0x7ff8000000000000LL);
-      }
-    }
-  }
+  const float pdivu_f = 0.5f * (Fxp[7] + Fxm[7]) * (Fxp[6] - Fxm[6]) * mk.idx0 +
+                        0.5f * (Fyp[7] + Fym[7]) * (Fyp[6] - Fym[6]) * mk.idx1 +
+                        0.5f * (Fzp[7] + Fzm[7]) * (Fzp[6] - Fzm[6]) * mk.idx2;
   const double pdivu = f2d_exact(pdivu_f);
-  const double rho = in.s[0];
-  const double m0 = in.s[1], m1 = in.s[2], m2 = in.s[3];
-  const double rE = in.s[4], re = in.s[5];
-  const double g0 = in.g[0], g1 = in.g[1], g2 = in.g[2];
+  const double rho = S[id];
+  const double m0 = S[bs + id], m1 = S[2 * bs + id], m2 = S[3 * bs + id];
+  const double rE = S[4 * bs + id], re = S[5 * bs + id];
+  double g0 = 0.0, g1 = 0.0, g2 = 0.0;
+  if (G) {
+    g0 = G[id];
+    g1 = G[bs + id];
+    g2 = G[2 * bs + id];
+  }
   const double rho_s = rho - sc.dtp * div[0];
   const double dtrho = sc.dt * rho;
   const double ms0 = (sc.a_old * m0 - sc.dt * div[1] + dtrho * g0) * sc.ian;
   const double ms1 = (sc.a_old * m1 - sc.dt * div[2] + dtrho * g1) * sc.ian;
   const double ms2 = (sc.a_old * m2 - sc.dt * div[3] + dtrho * g2) * sc.ian;
   // 1/rho: FP32 reciprocal, one Newton step in FP64 (relative error ~1e-14)
-  const float rho_f = (float)rho_s;
+  const float rho_f = d2f_rn(rho_s);
   double ir = f2d_exact(1.0f / rho_f);
   ir = ir * (2.0 - rho_s * ir);
   const double mg = m0 * g0 + m1 * g1 + m2 * g2;
   double rE_s;
-  if (genergy) {
+  if (k.grav_energy) {
     // Sec. 3.2, second alternative: the kinetic-energy change of the gravity update
     const double mh0 = (sc.a_old * m0 - sc.dt * div[1]) * sc.ian;
     const double mh1 = (sc.a_old * m1 - sc.dt * div[2]) * sc.ian;
@@ -328,7 +289,7 @@ __device__ __forceinline__ void update_cell_mixed(
     mn0 = ms0 + cr * g0;
     mn1 = ms1 + cr * g1;
     mn2 = ms2 + cr * g2;
-    if (genergy) {
+    if (k.grav_energy) {
       const double ks = ms0 * ms0 + ms1 * ms1 + ms2 * ms2;
       const double kn = mn0 * mn0 + mn1 * mn1 + mn2 * mn2;
       rEn = rE_s + 0.5 * (kn - ks) * ir;
@@ -362,13 +323,13 @@ __device__ __forceinline__ void update_cell_mixed(
   Sn[5 * bs + id] = ren;
   if (want_dt && full) {
     const float irf = 1.0f / rho_f;
-    float p = mk.gm1 * (float)ren;
+    float p = mk.gm1 * d2f_rn(ren);
     if (p < mk.small_pres) p = mk.small_pres;
     const float c2 = mk.gamma * p * irf;
     const float c = c2 * rsqrtf(c2);
-    const float t0 = mk.an_dx0 / (fabsf((float)mn0 * irf) + c);
-    const float t1 = mk.an_dx1 / (fabsf((float)mn1 * irf) + c);
-    const float t2 = mk.an_dx2 / (fabsf((float)mn2 * irf) + c);
+    const float t0 = mk.an_dx0 / (fabsf(d2f_rn(mn0) * irf) + c);
+    const float t1 = mk.an_dx1 / (fabsf(d2f_rn(mn1) * irf) + c);
+    const float t2 = mk.an_dx2 / (fabsf(d2f_rn(mn2) * irf) + c);
     dtmin = fminf(dtmin, fminf(t0, fminf(t1, t2)));
   }
 }
@@ -664,12 +625,8 @@ __global__ void __launch_bounds__(FusedGeom<R, TX, TY>::NT, 1) k_fused(nyx::Fuse
         const long long id = col + (long long)(c - 1 + 4) * ps;
         if constexpr (sizeof(R) == 4) {
           float dtf = __int_as_float(0x7f800000);
-          auto flux = [&](int k, int f) {
-            return f == 0 ? Fxm[k] : f == 1 ? Fxp[k] : f == 2 ? Fym[k] : f == 3 ? Fyp[k]
-                 : f == 4 ? Ffz_prev[k] : Ffz[k];
-          };
-          update_cell_mixed(KK, sc, bs, mixk, load_cell(S, G, bs, id), Sn, id, flux, dtf,
-                            flags, a.dtacc != nullptr, !a.predict_only, false, KK.grav_energy != 0);
+          update_cell_mixed(KK, sc, b, mixk, S, G, Sn, id, Fxm, Fxp, Fym, Fyp, Ffz_prev, Ffz, dtf,
+                            flags, a.dtacc != nullptr, !a.predict_only);
           if ((double)dtf < dtmin) dtmin = (double)dtf;
         } else
           update_cell<R>(KK, sc, b, S, G, Sn, id, Fxm, Fxp, Fym, Fyp, Ffz_prev, Ffz, dtmin, flags,

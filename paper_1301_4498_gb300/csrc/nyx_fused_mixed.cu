@@ -16,17 +16,15 @@ int launch_fused_mixed(int shape, const FusedArgs &a, int grid, cudaStream_t st)
     case 0: return nyx_mixed::launch_one<float, 16, 16>(a, grid, st);
     case 1: return nyx_mixed::launch_one<float, 32, 8>(a, grid, st);
     case 2: return nyx_mixed::launch_one<float, 16, 8>(a, grid, st);
-    case 3:  // the default shape: one instantiation per scheme variant in common use, the
-             // others take the one with run-time variant flags
+    case 3:  // the default shape: one instantiation per scheme variant (flattening with
+             // PLM or the linearised solver: the one with run-time variant flags)
+      if (a.variant == 4) return nyx_mixed::launch_two<16, 8, 1, 4>(a, grid, st);
+      if (a.variant & 4) return nyx_mixed::launch_two<16, 8, 1, -1>(a, grid, st);
       switch (a.variant) {
-        case 0: return nyx_mixed::launch_two<16, 8, 1, 0>(a, grid, st);
         case 1: return nyx_mixed::launch_two<16, 8, 1, 1>(a, grid, st);
         case 2: return nyx_mixed::launch_two<16, 8, 1, 2>(a, grid, st);
         case 3: return nyx_mixed::launch_two<16, 8, 1, 3>(a, grid, st);
-        case 4: return nyx_mixed::launch_two<16, 8, 1, 4>(a, grid, st);
-        case 8: return nyx_mixed::launch_two<16, 8, 1, 8>(a, grid, st);
-        case 12: return nyx_mixed::launch_two<16, 8, 1, 12>(a, grid, st);
-        default: return nyx_mixed::launch_two<16, 8, 1, -1>(a, grid, st);
+        default: return nyx_mixed::launch_two<16, 8, 1, 0>(a, grid, st);
       }
     case 4: return nyx_mixed::launch_two<8, 8, 2, -1>(a, grid, st);
     case 5: return nyx_mixed::launch_two<32, 4, 1, -1>(a, grid, st);
@@ -45,8 +43,6 @@ int max_grid_mixed(int shape) {
       g = std::min(g, nyx_mixed::max_grid_two<16, 8, 1, 2>());
       g = std::min(g, nyx_mixed::max_grid_two<16, 8, 1, -1>());
       g = std::min(g, nyx_mixed::max_grid_two<16, 8, 1, 4>());
-      g = std::min(g, nyx_mixed::max_grid_two<16, 8, 1, 8>());
-      g = std::min(g, nyx_mixed::max_grid_two<16, 8, 1, 12>());
       return std::min(g, nyx_mixed::max_grid_two<16, 8, 1, 3>());
     }
     case 4: return nyx_mixed::max_grid_two<8, 8, 2, -1>();
