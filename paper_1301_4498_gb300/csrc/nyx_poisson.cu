@@ -560,6 +560,9 @@ struct FastDiv {
 constexpr int kTailMax = 12;        // grids in the list
 constexpr int kTailCells = 8192;    // cells of its largest grid (one CTA's work)
 constexpr int kTailThreads = 512;
+// phi and f of all its grids, each at most an eighth of the one above it
+template <class T>
+constexpr size_t kTailSmem = 2 * sizeof(T) * (kTailCells + kTailCells / 7);
 template <class T>
 struct TailArgs {
   int n;                 // grids
@@ -1026,8 +1029,10 @@ size_t make_tail(const nyx_poisson *S, const std::vector<LevelT<T>> &L, size_t f
   a.f = L[t].f;
   a.phi = L[t].phi;
   smem = sizeof(T) * (size_t)off;
-  if (cudaFuncSetAttribute(k_pg_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess) {
+  // the attribute is the kernel's, shared by every solver alive: set to what
+  // the largest tail takes, never to this one's own size
+  if (cudaFuncSetAttribute(k_pg_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kTailSmem<T>) != cudaSuccess) {
     cudaGetLastError();
     return L.size();
   }
@@ -1371,6 +1376,7 @@ static int run_cycles(nyx_poisson *S, double target, int *cyc, double *res) {
     if (int rc = resid_max(S, res)) return rc;
   while (*res > target && *cyc < S->prm.max_cycles) {
     cycle(S);
+    CK(cudaGetLastError());  // a launch that failed ends the solve here
     ++*cyc;
     if (int rc = resid_max(S, res)) return rc;
   }

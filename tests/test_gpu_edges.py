@@ -190,3 +190,44 @@ def test_mixed_poisson_solve(n, prm, scale, warm):
     assert np.abs(phi - ref).max() <= 0.26 * tol * np.abs(f).max() + 1e-12 * np.abs(ref).max()
     ps.close()
     plan.close()
+
+
+def _poisson_box(n, seed, **prm):
+    """(plan, solver, device state, spectral potential of its density, max|f|)
+    of one periodic box of n = (nx, ny, nz) cells of width 1 / max(n)."""
+    h = 1.0 / max(n)
+    lev = W.single_box_level(*n, h)
+    arr = np.zeros(lev.shape(0, 6))
+    rho = np.exp(np.random.default_rng(seed).standard_normal(n[::-1]))
+    W.valid(arr)[0] = rho
+    plan = H.Plan(lev, precision="fp64")
+    f = rho - rho.mean()
+    return (plan, H.Poisson(plan, **prm), plan.to_device([arr], 6), _spectral_phi(f, h),
+            np.abs(f).max())
+
+
+def _solve_and_check(box, tol, warm=False):
+    _, ps, state, ref, fmax = box
+    cyc, res = ps.solve(state, 1.0, None, warm_start=warm)
+    phi = ps.phi().cpu().numpy()
+    # the bound of test_mixed_poisson_solve, l = 1
+    assert res <= tol
+    assert (np.abs(phi - phi.mean() - ref).max()
+            <= 0.26 * tol * fmax + 1e-12 * np.abs(ref).max())
+    return cyc, res
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("first,second", [(128, 96), (96, 128), (40, 128)])
+def test_live_solvers_keep_their_own_tails(first, second, precision):
+    # the coarse grids run in one CTA whose shared memory differs by grid: a
+    # solver made later, or destroyed, must not narrow what an earlier one may use
+    a = _poisson_box((first,) * 3, 1, precision=precision, tol=1e-11)
+    b = _poisson_box((second,) * 3, 2, precision=precision, tol=1e-11)
+    for box in (a, b, a):
+        _solve_and_check(box, 1e-11)
+    b[1].close()
+    _solve_and_check(a, 1e-11)
+    a[1].close()
+    a[0].close()
+    b[0].close()
