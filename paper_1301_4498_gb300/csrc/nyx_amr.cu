@@ -288,6 +288,7 @@ struct nyx_amr {
   int n_avg = 0;
   unsigned char *d_cov = nullptr;
   std::map<AmrKey, std::pair<cudaGraphExec_t, long long>> graphs;
+  std::pair<long long, long long> graphs_gen{0, 0};  // the plans' shape_gen they are of
 };
 
 namespace {
@@ -787,6 +788,13 @@ int nyx_amr_run(nyx_amr *A, nyx_level *Lc, nyx_level *Lf, const double *a_dev, d
     if ((rc = enqueue_interp(A, Lc->state[Lc->cur], Lf->state[Lf->cur], NCONS, NYX_AMR_GHOSTS)))
       return rc;
     if ((rc = plan_tune(&F, Lf, a_dev, dt_dev))) return rc;
+  }
+  const std::pair<long long, long long> gen(C.shape_gen, F.shape_gen);
+  if (A->graphs_gen != gen) {  // recorded with another tile shape
+    CK(cudaStreamSynchronize(C.stream));
+    for (auto &kv : A->graphs) cudaGraphExecDestroy(kv.second.first);
+    A->graphs.clear();
+    A->graphs_gen = gen;
   }
   AmrKey key(Lc->state[0], Lc->state[1], Lf->state[0], Lf->state[1], Lc->grav, Lf->grav,
              Lc->cur * 2 + Lf->cur, a_dev, dt_dev, nsteps, compute_dt0);

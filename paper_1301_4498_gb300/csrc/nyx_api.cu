@@ -496,10 +496,11 @@ void free_plan(nyx_plan *P) {
   cudaFree(P->d_flux_off);
   for (auto &it : P->d_items) cudaFree(it);
   for (auto &it : P->d_items_grp) cudaFree(it);
-  for (auto &pt : P->parts) {
-    cudaFree(pt.d_items);
-    cudaFree(pt.d_items_grp);
-  }
+  for (auto *v : {&P->parts, &P->old_parts})
+    for (auto &pt : *v) {
+      cudaFree(pt.d_items);
+      cudaFree(pt.d_items_grp);
+    }
   for (auto &e : P->ev_grp) cudaEventDestroy(e);
   for (auto &kv : P->tmaps) cudaFree(kv.second);
   if (P->copy_stream) cudaStreamDestroy(P->copy_stream);
@@ -1136,6 +1137,14 @@ std::vector<WorkItem> subset_items(const nyx_plan &P, const std::vector<int> &se
   return it;
 }
 
+// Another shape, or other parts, from here on.
+void change_shape(nyx_plan *P, int shape) {
+  for (auto &pt : P->parts) P->old_parts.push_back(std::move(pt));
+  P->parts.clear();
+  P->shape = shape;
+  ++P->shape_gen;
+}
+
 int tune_shape(nyx_plan *P, const FusedArgs &base) {
   P->tuned = true;
   cudaStreamCaptureStatus cs;
@@ -1257,15 +1266,10 @@ int tune_shape(nyx_plan *P, const FusedArgs &base) {
     gcells[{pick[c].shape, pick[c].per_sm}] +=
         (long long)cls_boxes[c].size() * cls_n[c][0] * cls_n[c][1] * cls_n[c][2];
   }
-  for (auto &pt : P->parts) {
-    cudaFree(pt.d_items);
-    cudaFree(pt.d_items_grp);
-  }
-  P->parts.clear();
   auto biggest = gcells.begin();
   for (auto it = gcells.begin(); it != gcells.end(); ++it)
     if (it->second > biggest->second) biggest = it;
-  P->shape = biggest->first.first;
+  change_shape(P, biggest->first.first);
   if (groups.size() == 1 && biggest->first.second * nsm >= P->max_grid[P->shape])
     return ensure_items(P, P->shape);
   for (auto &kv : groups) {
@@ -1811,6 +1815,12 @@ int nyx_hydro_run(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev
     if (rc) return rc;
   }
   if (P->prm.batching == NYX_PERSISTENT) prepare_tmaps(P, L);
+  if (P->graphs_gen != P->shape_gen) {  // recorded with another shape
+    CK(cudaStreamSynchronize(P->stream));
+    for (auto &kv : P->graphs) cudaGraphExecDestroy(kv.second.first);
+    P->graphs.clear();
+    P->graphs_gen = P->shape_gen;
+  }
   GraphKey key(L->state[0], L->state[1], L->grav, L->cur, a_dev, dt_dev, nsteps, compute_dt0);
   auto it = P->graphs.find(key);
   if (it == P->graphs.end()) {
@@ -1988,12 +1998,7 @@ int nyx_hydro_set_tile_shape(nyx_plan *P, int shape) {
   if (P->prm.batching != NYX_PERSISTENT) return fail(NYX_EINVAL, "plan is not persistent");
   if (shape < 0 || shape >= fused_num_shapes(P->prm.precision)) return fail(NYX_EINVAL, "tile shape out of range");
   if (int rc = ensure_items(P, shape)) return rc;
-  for (auto &pt : P->parts) {
-    cudaFree(pt.d_items);
-    cudaFree(pt.d_items_grp);
-  }
-  P->parts.clear();
-  P->shape = shape;
+  if (shape != P->shape || !P->parts.empty()) change_shape(P, shape);
   P->tuned = true;
   return NYX_OK;
 }

@@ -130,6 +130,12 @@ struct nyx_plan {
     std::vector<int> grp_off;  // first item of each read-back group, ngrp + 1 entries
   };
   std::vector<RunPart> parts;
+  // parts given up for another shape: graphs recorded earlier, the plan's own
+  // or a caller's, may still hold their lists, so these live as long as the
+  // plan (only tuning makes parts, once per plan)
+  std::vector<RunPart> old_parts;
+  // counts the changes of shape or parts; cached graphs are of graphs_gen
+  long long shape_gen = 0, graphs_gen = 0;
   // TMA descriptors of level fields for the shapes that stage with tensor
   // copies: one CUtensorMap per box, in device memory, keyed by (field
   // address, components, shape); null marks a field that cannot be mapped
