@@ -368,23 +368,31 @@ __device__ __forceinline__ float d2f_trunc(double v) {
 // float (the right-hand side of the FP32 correction solve), the max norm of
 // that float residual, and the correction's start e = 0.  The Laplacian is
 // formed as f + 6 ih2 phi - ih2 (sum of the neighbours) with two fused
-// multiply-adds: 7 FP64 operations per cell (c6 = 6 ih2).
+// multiply-adds: 7 FP64 operations per cell (c6 = 6 ih2).  With pmax, also
+// max |phi| (a NaN's bits lie above all others).
 // (grid3 of (n_x, n_y, n_z))
 __global__ void k_pg_resid32(const double *phi, const double *f, Dims d, double ih2, double c6,
-                             float *r, float *e, unsigned long long *out) {
+                             float *r, float *e, unsigned long long *out,
+                             unsigned long long *pmax) {
   float loc = 0.0f;
+  unsigned long long pm = 0;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < d.n[0]) {
     const int j = blockIdx.y, k = blockIdx.z;
     const long long t = didx(d, i, j, k);
-    const double v = fma(-ih2, nbsum(phi, d, i, j, k), fma(c6, phi[t], f[t]));
+    const double u = phi[t];
+    const double v = fma(-ih2, nbsum(phi, d, i, j, k), fma(c6, u, f[t]));
     const float v32 = d2f_trunc(v);
+    pm = (unsigned long long)__double_as_longlong(u) & ~(1ull << 63);
     r[t] = v32;
     e[t] = 0.0f;
     loc = fabsf(v32);
   }
   for (int o = 16; o > 0; o >>= 1) loc = fmaxf(loc, __shfl_xor_sync(0xffffffffu, loc, o));
   if ((threadIdx.x & 31) == 0) atomic_max_pos(out, (double)loc);
+  if (!pmax) return;
+  for (int o = 16; o > 0; o >>= 1) pm = max(pm, __shfl_xor_sync(0xffffffffu, pm, o));
+  if ((threadIdx.x & 31) == 0) atomic_max_pos(pmax, __longlong_as_double((long long)pm));
 }
 
 // phi += e (the FP32 correction), in FP64
@@ -396,13 +404,18 @@ __global__ void k_pg_correct(double *phi, const float *e, long long n) {
 
 // ---------------------------------------------------------------- fixed point
 // The refinement solve's potential and right-hand side as 64-bit integers: phi
-// in units of 1/s, s a power of two that puts a bound of every potential the
-// solve can meet near 2^62, and h^2 f in units of 1/(s 2^K), K what its own
-// maximum leaves (it is smaller than the potential by up to n^2).  The
-// residual's seven terms then add exactly (modulo 2^64) on the integer pipe,
-// and phi += e loses nothing but e's own last bits, while in FP64 the
-// residual's 7 operations a cell alone take this part's FP64 pipe 187 us on a
-// 256^3 grid and round at 2^-53 of the potential.
+// in units of 1/s, s a power of two that puts a bound of the solution in
+// [2^59, 2^60), and h^2 f in units of 1/(s 2^K), K what its own maximum leaves
+// (it is smaller than the potential by up to n^2).  The residual's seven terms
+// then add exactly (modulo 2^64) on the integer pipe, and phi += e loses
+// nothing but e's own last bits, while in FP64 the residual's 7 operations a
+// cell alone take this part's FP64 pipe 187 us on a 256^3 grid.
+//
+// The first bound comes from the right-hand side alone and may lie 2^13 (a
+// 256^3 grid) and more above the potential; as the residual falls it closes in
+// (refine_fixed), and phi moves to a finer unit, b bits by a shift, with K - b
+// for K: h^2 f stays as it is.  At the end phi's unit is about 2^-59 of its
+// maximum.  Rounding phi to units leaves a residual of about 6 units / h^2.
 
 // float -> fixed, nearest: |e s| as hi 2^32 + lo, both exact in FP32 (a
 // negative number's low half, 2^32 - x, would not be)
@@ -444,21 +457,15 @@ __global__ void k_pg_from_fix(const long long *y, double *x, long long n, double
        t += (long long)gridDim.x * blockDim.x)
     x[t] = (double)y[t] * is;
 }
-__global__ void k_pg_absmax(const double *x, long long n, unsigned long long *out) {
-  unsigned long long loc = 0;
+__global__ void k_pg_shift_fix(long long *y, long long n, int b) {
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-       t += (long long)gridDim.x * blockDim.x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x[t]) & ~(1ull << 63);
-    loc = loc > b ? loc : b;
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long b = __shfl_xor_sync(0xffffffffu, loc, o);
-    loc = loc > b ? loc : b;
-  }
-  if ((threadIdx.x & 31) == 0) atomic_max_pos(out, __longlong_as_double((long long)loc));
+       t += (long long)gridDim.x * blockDim.x)
+    y[t] = (long long)((unsigned long long)y[t] << b);
 }
 
-// Residual r = f - L phi of the finest grid as float, and the max norm of it.
+// Residual r = f - L phi of the finest grid as float, the max norm of it
+// (out[0]) and the high word of the largest |phi| (out[1]; |phi| is at most
+// (out[1] + 1) 2^32 units).
 // h^2 r = f 2^-K + 6 phi - (neighbours) keeps f's K extra bits where the sum of
 // the others leaves room for them (|.| < 2^(62-K)), else they are below its
 // rounding to float; c = 1 / (h^2 s).
@@ -488,6 +495,7 @@ __global__ void __launch_bounds__(kRfX *kRfY)
     return q;
   };
   float loc = 0.0f;
+  unsigned pm = 0;
   const int nx = d.n[0], ny = d.n[1], nz = d.n[2];
   const int i = (blockIdx.x * kRfX + threadIdx.x) * W, j = blockIdx.y * kRfY + threadIdx.y;
   const int z0 = blockIdx.z * zc, z1 = min(nz, z0 + zc);
@@ -516,6 +524,8 @@ __global__ void __launch_bounds__(kRfX *kRfY)
         const unsigned long long x = fine ? (v << K) + (unsigned long long)(F & ((1ll << K) - 1)) : v;
         q[u] = from_fix((long long)x) * (fine ? cK : c);
         loc = fmaxf(loc, fabsf(q[u]));
+        const int top = (int)(mid.v[u] >> 32);
+        pm = max(pm, (unsigned)(top ^ (top >> 31)));
       }
       if (PAIR)
         *reinterpret_cast<float2 *>(r + zb + o) = make_float2(q[0], q[W - 1]);
@@ -526,7 +536,12 @@ __global__ void __launch_bounds__(kRfX *kRfY)
     }
   }
   for (int o = 16; o > 0; o >>= 1) loc = fmaxf(loc, __shfl_xor_sync(0xffffffffu, loc, o));
-  if (threadIdx.x == 0) atomic_max_pos(out, (double)loc);
+  pm = __reduce_max_sync(0xffffffffu, pm);
+  if (threadIdx.x == 0) {
+    atomic_max_pos(out, (double)loc);
+    if (pm > *reinterpret_cast<volatile unsigned long long *>(out + 1))
+      atomicMax(out + 1, (unsigned long long)pm);
+  }
 }
 
 __global__ void k_pg_correct_fix(long long *phi, const float *e, long long n, float s) {
@@ -948,12 +963,13 @@ struct nyx_poisson {
   TailArgs<float> targs32{};
   size_t tsmem64 = 0, tsmem32 = 0;
   // fixed-point potential of the refinement solve (while `fixed`): units of
-  // 1/fix_s; h^2 times the right-hand side is then fixed point in L[0].f's
-  // memory, in units of 1/(fix_s 2^fix_k)
+  // 1/fix_s, at most (fix_top + 1) 2^32 of them; h^2 times the right-hand side
+  // is then fixed point in L[0].f's memory, in units of 1/(fix_s 2^fix_k)
   long long *d_fix = nullptr;
   bool fixed = false;
   float fix_s = 0.0f;
   int fix_k = 0;
+  unsigned fix_top = 0;
 };
 
 namespace {
@@ -978,11 +994,13 @@ void free_poisson(nyx_poisson *S) {
   delete S;
 }
 
-int read_max(nyx_poisson *S, double *out) {
-  unsigned long long v = 0;
-  CK(cudaMemcpyAsync(&v, S->d_max, sizeof(v), cudaMemcpyDeviceToHost, S->P->stream));
+int read_max(nyx_poisson *S, double *out, unsigned long long *second = nullptr) {
+  unsigned long long v[2] = {0, 0};
+  CK(cudaMemcpyAsync(v, S->d_max, (second ? 2 : 1) * sizeof(v[0]), cudaMemcpyDeviceToHost,
+                     S->P->stream));
   CK(cudaStreamSynchronize(S->P->stream));
-  std::memcpy(out, &v, sizeof(double));
+  std::memcpy(out, v, sizeof(double));
+  if (second) *second = v[1];
   return NYX_OK;
 }
 
@@ -1179,9 +1197,12 @@ void vcycle_fused(nyx_poisson *S) {
 
 bool fused_cycle(const nyx_poisson *S) { return S->prm.pre >= 1 && S->prm.post >= 1; }
 
-int resid_max(nyx_poisson *S, double *out) {
+// Max norm of the finest grid's residual, and with pmax (mixed precision, phi
+// in FP64) the largest |phi|.
+int resid_max(nyx_poisson *S, double *out, double *pmax = nullptr) {
   Level &g = S->L[0];
-  CK(cudaMemsetAsync(S->d_max, 0, sizeof(unsigned long long), S->P->stream));
+  unsigned long long second = 0;
+  CK(cudaMemsetAsync(S->d_max, 0, 2 * sizeof(unsigned long long), S->P->stream));
   if (S->fixed) {
     LevelT<float> &g32 = S->L32[0];
     const int w = g.d.n[0] % 2 ? 1 : 2;
@@ -1199,10 +1220,53 @@ int resid_max(nyx_poisson *S, double *out) {
     LevelT<float> &g32 = S->L32[0];
     const Grid3 G = grid3(g.d.n[0], g.d.n[1], g.d.n[2]);
     k_pg_resid32<<<G.g, G.b, 0, S->P->stream>>>(g.phi, g.f, g.d, g.ih2, 6.0 * g.ih2, g32.f,
-                                                g32.phi, S->d_max);
+                                                g32.phi, S->d_max, pmax ? S->d_max + 1 : nullptr);
   }
   S->launches += 1;
-  return read_max(S, out);
+  if (int rc = read_max(S, out, S->fixed || pmax ? &second : nullptr)) return rc;
+  if (S->fixed) S->fix_top = (unsigned)second;
+  if (pmax) std::memcpy(pmax, &second, sizeof(double));
+  return NYX_OK;
+}
+
+// Largest |e| that a zero-mean residual of max norm r can still call for (L e =
+// r) on a periodic box of longest side l: 0.26 l^2 r, by Cauchy-Schwarz over its
+// Fourier modes, whose discrete eigenvalues are at least 4 / pi^2 of k^2.
+double correction_bound(const nyx_poisson *S, double r) {
+  const Dims &d = S->L[0].d;
+  const double side = std::max(d.n[0], std::max(d.n[1], d.n[2])) * S->dx;
+  return 0.26 * side * side * r;
+}
+
+// smallest e with x < 2^e
+int exponent(double x) {
+  int e = 0;
+  std::frexp(x, &e);
+  return e;
+}
+
+bool fix_scale_ok(const nyx_poisson *S, double s) {  // FP32 holds s and the residual's scale
+  const double c = S->L[0].ih2 / s;
+  return s < 1e36 && c > 1e-27 && c < 1e30;
+}
+
+// A finer unit for the fixed-point potential, once what its bound leaves unused
+// is worth a pass (16 B a cell): when the measured potential makes up most of
+// the bound (from there on little is to be gained by waiting), or when the
+// residual (res) is within 4096 units of being lost in them.
+void refine_fixed(nyx_poisson *S, double res) {
+  const Level &g = S->L[0];
+  const double s = S->fix_s;
+  const double pm = ((double)S->fix_top + 1.0) * 4294967296.0, left = correction_bound(S, res) * s;
+  if (left > pm && g.h2 * res * s > 4096.0) return;
+  int b = std::min(60 - exponent(pm + left), S->fix_k);
+  while (b > 0 && !fix_scale_ok(S, std::ldexp(s, b))) --b;
+  if (b < 2) return;
+  const long long n = (long long)g.d.n[0] * g.d.n[1] * g.d.n[2];
+  k_pg_shift_fix<<<gridn(n, 256), 256, 0, S->P->stream>>>(S->d_fix, n, b);
+  S->launches += 1;
+  S->fix_s = (float)std::ldexp(s, b);
+  S->fix_k -= b;
 }
 
 // One cycle: a V-cycle on phi (FP64), or a refinement step (FP32 V-cycle on
@@ -1375,6 +1439,7 @@ static int run_cycles(nyx_poisson *S, double target, int *cyc, double *res) {
   if (*res < 0.0)
     if (int rc = resid_max(S, res)) return rc;
   while (*res > target && *cyc < S->prm.max_cycles) {
+    if (S->fixed) refine_fixed(S, *res);
     cycle(S);
     CK(cudaGetLastError());  // a launch that failed ends the solve here
     ++*cyc;
@@ -1383,34 +1448,32 @@ static int run_cycles(nyx_poisson *S, double target, int *cyc, double *res) {
   return NYX_OK;
 }
 
-// Start the solve in fixed point if a scale fits: the potential of a zero-mean
-// right-hand side of max norm fmax on a periodic box of longest side l is at
-// most 0.26 l^2 fmax (Cauchy-Schwarz over its Fourier modes, whose discrete
-// eigenvalues are at least 4 / pi^2 of k^2), and the start's own potential is
-// measured.  The sum of the first and 8 of the second is kept below 2^61: six
-// times any difference of two potentials then stays below 2^63.  A start from
-// phi = 0 leaves its residual, f, and the norm of it.
-static int start_fixed(nyx_poisson *S, double fmax, int warm, double *res) {
+// Start the solve in fixed point if a scale fits.  The solution is at most the
+// start's largest |phi| and the correction that its residual calls for; s puts
+// that in [2^59, 2^60), and h^2 f below 2^61.  A potential on the way exceeds the
+// bound by no more than a residual that grows instead of falling calls for, and
+// the residual's sum, h^2 r whatever the size of its terms, by no more either:
+// both have a factor of 8 to the int64's limit.
+// A start from phi = 0 leaves its residual, f, and the norm of it.  A given
+// potential's residual is formed in FP64, and the potential is left as it is
+// where that meets the target.
+static int start_fixed(nyx_poisson *S, double fmax, int warm, double target, double *res) {
   Level &g = S->L[0];
   const long long n = (long long)g.d.n[0] * g.d.n[1] * g.d.n[2];
   cudaStream_t st = S->P->stream;
   double pmax = 0.0;
   if (warm) {
-    CK(cudaMemsetAsync(S->d_max, 0, sizeof(unsigned long long), st));
-    k_pg_absmax<<<gridn(n, 256), 256, 0, st>>>(g.phi, n, S->d_max);
-    S->launches += 1;
-    if (int rc = read_max(S, &pmax)) return rc;
+    if (int rc = resid_max(S, res, &pmax)) return rc;
+    if (*res <= target) return NYX_OK;
   }
-  const double side = std::max(g.d.n[0], std::max(g.d.n[1], g.d.n[2])) * S->dx;
-  const double bound = 2.0 * (0.26 * side * side * fmax + 8.0 * pmax);
+  const double bound = pmax + correction_bound(S, warm ? *res : fmax);
   if (!(bound > 1e-15 && bound < 1e15)) return NYX_OK;  // FP64 residuals instead
-  const double s = std::ldexp(1.0, 62 - (int)std::ceil(std::log2(bound)));
-  // the residual's scale stays inside FP32's range
-  const double c = g.ih2 / s;
-  if (!(c > 1e-27 && c < 1e30 && s < 1e36)) return NYX_OK;
-  const double hf = g.h2 * s * fmax;  // in (0, 2^61): h^2 f < bound / 2
-  S->fix_k = std::min(31, 61 - (hf > 1.0 ? (int)std::ceil(std::log2(hf)) : 0));
+  const int es = 60 - exponent(bound), ef = fmax > 0.0 ? 61 - exponent(g.h2 * fmax) : es;
+  const double s = std::ldexp(1.0, std::min(es, ef));
+  if (!fix_scale_ok(S, s)) return NYX_OK;
+  S->fix_k = std::min(31, ef - std::min(es, ef));
   S->fix_s = (float)s;
+  S->fix_top = (unsigned)(pmax * s / 4294967296.0);
   S->fixed = true;
   k_pg_rhs_fix<<<gridn(n, 256), 256, 0, st>>>(g.f, (long long *)g.f, n,
                                               std::ldexp(g.h2 * s, S->fix_k), S->d_fix,
@@ -1439,7 +1502,7 @@ int nyx_poisson_solve(nyx_poisson *S, const double *state, const double *rho_dm,
   int rc = build_rhs(S, state, rho_dm, a, &fmax);
   if (rc) return rc;
   const double target = S->prm.tol * fmax;
-  if (S->d_fix && (rc = start_fixed(S, fmax, warm_start, &res))) return rc;
+  if (S->d_fix && (rc = start_fixed(S, fmax, warm_start, target, &res))) return rc;
   if (S->fixed) {
     rc = run_cycles(S, target, &cyc, &res);
     S->fixed = false;

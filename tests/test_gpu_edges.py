@@ -231,3 +231,41 @@ def test_live_solvers_keep_their_own_tails(first, second, precision):
     a[1].close()
     a[0].close()
     b[0].close()
+
+
+def test_mixed_poisson_at_tolerances_near_rounding():
+    # an uncorrelated density: FP64 sums leave a residual of about 1e-16 max|f|
+    box = _poisson_box((128,) * 3, 3, precision="mixed", tol=2e-15, max_cycles=30)
+    _solve_and_check(box, 2e-15)
+    # the same density again: solved already, and left as it is
+    before = box[1].phi()
+    assert _solve_and_check(box, 2e-15, warm=True)[0] == 0
+    assert torch.equal(before, box[1].phi())
+    box[1].close()
+    box[0].close()
+
+
+@pytest.mark.parametrize("warm", [False, True])
+def test_mixed_poisson_on_a_long_domain(warm):
+    # 2048 x 16 x 16 cells at the default tolerance, a density of period 32
+    # cells (so that it converges as one period does): the potential is 64^2
+    # times smaller than a domain of this length allows
+    n, h, per = (2048, 16, 16), 1.0 / 2048, 32
+    rng = np.random.default_rng(8)
+    cell = [np.exp(rng.standard_normal((16, 16, per))) for _ in range(2)]
+    lev = W.single_box_level(*n, h)
+    plan = H.Plan(lev, precision="fp64")
+    ps = H.Poisson(plan, precision="mixed")
+    for c in cell[:1 + warm]:
+        arr = np.zeros(lev.shape(0, 6))
+        W.valid(arr)[0] = np.tile(c, (1, 1, n[0] // per))
+        cyc, res = ps.solve(plan.to_device([arr], 6), 1.0, None, warm_start=warm)
+        assert res <= 1e-12
+    f = c - c.mean()
+    ref = np.tile(_spectral_phi(f, h), (1, 1, n[0] // per))
+    phi = ps.phi().cpu().numpy()
+    # (of length 32 h each period)
+    assert (np.abs(phi - phi.mean() - ref).max()
+            <= 0.26 * (per * h)**2 * 1e-12 * np.abs(f).max() + 1e-12 * np.abs(ref).max())
+    ps.close()
+    plan.close()
