@@ -442,12 +442,13 @@ int ensure_items(nyx_plan *P, int s) {
     return e;
   };
   cudaError_t e = cudaSuccess;
-  if (P->ngrp > 1) {  // box groups are set up already: this shape's items by group
+  for (auto &B : P->groups) {  // set up already: this shape's items by group too
+    if (B.n < 2 || B.items[s].d || e != cudaSuccess) continue;
     std::vector<WorkItem> by;
     std::vector<int> off(1, 0);
-    group_items(it, P->grp_box, by, off);
-    e = upload(by, &P->d_items_grp[s]);
-    if (e == cudaSuccess) P->grp_off[s] = off;
+    group_items(it, B.box, by, off);
+    e = upload(by, &B.items[s].d);
+    if (e == cudaSuccess) B.items[s].off = off;
   }
   if (e == cudaSuccess) e = upload(it, &P->d_items[s]);
   cudaThreadExchangeStreamCaptureMode(&mode);
@@ -495,17 +496,20 @@ void free_plan(nyx_plan *P) {
   cudaFree(P->d_flux);
   cudaFree(P->d_flux_off);
   for (auto &it : P->d_items) cudaFree(it);
-  for (auto &it : P->d_items_grp) cudaFree(it);
   for (auto *v : {&P->parts, &P->old_parts})
     for (auto &pt : *v) {
       cudaFree(pt.d_items);
-      cudaFree(pt.d_items_grp);
+      for (auto &g : pt.grp) cudaFree(g.d);
     }
-  for (auto &e : P->ev_grp) cudaEventDestroy(e);
+  for (auto &B : P->groups) {
+    for (auto &it : B.items) cudaFree(it.d);
+    for (auto &r : B.d_rects) cudaFree(r);
+    cudaFree(B.d_queue);
+    for (auto &e : B.ev_ready) cudaEventDestroy(e);
+    for (auto &e : B.ev_done) cudaEventDestroy(e);
+  }
   for (auto &kv : P->tmaps) cudaFree(kv.second);
   if (P->copy_stream) cudaStreamDestroy(P->copy_stream);
-  for (auto &r : P->d_rects_grp) cudaFree(r);
-  for (auto &e : P->ev_in) cudaEventDestroy(e);
   if (P->ev_start) cudaEventDestroy(P->ev_start);
   if (P->h2d_stream) cudaStreamDestroy(P->h2d_stream);
   if (P->ev_setup) cudaEventDestroy(P->ev_setup);
@@ -515,9 +519,6 @@ void free_plan(nyx_plan *P) {
     if (P->fill_stream[k]) cudaStreamDestroy(P->fill_stream[k]);
     if (P->ev_fjoin[k]) cudaEventDestroy(P->ev_fjoin[k]);
   }
-  for (auto &e : P->ev_gfill) cudaEventDestroy(e);
-  for (auto &e : P->ev_gadv) cudaEventDestroy(e);
-  cudaFree(P->d_queue_grp);
   cudaFree(P->d_queue);
   delete P;
 }
@@ -527,6 +528,8 @@ bool capturing(nyx_plan *P) {
   cudaStreamIsCapturing(P->stream, &cs);
   return cs != cudaStreamCaptureStatusNone;
 }
+
+bool untuned(const nyx_plan *P) { return P->prm.autotune && !P->tuned; }
 
 // Event pair around a span of launches when profiling an eager call.
 struct Span {
@@ -706,18 +709,21 @@ void set_tmaps(nyx_plan *P, FusedArgs &a, int shape) {
   if (!a.tmS || (a.G && !a.tmG)) a.tmS = a.tmG = nullptr;
 }
 
-// The fused advance over the whole level (g < 0) or over read-back group g:
-// one launch of the plan's shape, or one per part of the autotuner's
-// per-class choice.
-int launch_level(nyx_plan *P, FusedArgs a, int g, cudaStream_t st) {
+// The fused advance over the whole level (g < 0) or over group g of set w
+// (kHost or kRun): one launch of the plan's shape, or one per part of the
+// autotuner's per-class choice.
+int launch_level(nyx_plan *P, FusedArgs a, int w, int g, cudaStream_t st) {
+  const auto group = [&](const nyx_plan::GroupItems &v) {
+    a.items = v.d + v.off[g];
+    a.nitems = v.off[g + 1] - v.off[g];
+  };
   if (P->parts.empty()) {
     const int s = P->shape;
     if (g < 0) {
       a.items = P->d_items[s];
       a.nitems = P->nitems[s];
     } else {
-      a.items = P->d_items_grp[s] + P->grp_off[s][g];
-      a.nitems = P->grp_off[s][g + 1] - P->grp_off[s][g];
+      group(P->groups[w].items[s]);
     }
     if (a.nitems > 0) {
       set_tmaps(P, a, s);
@@ -732,8 +738,7 @@ int launch_level(nyx_plan *P, FusedArgs a, int g, cudaStream_t st) {
       a.items = pt.d_items;
       a.nitems = pt.nitems;
     } else {
-      a.items = pt.d_items_grp + pt.grp_off[g];
-      a.nitems = pt.grp_off[g + 1] - pt.grp_off[g];
+      group(pt.grp[w]);
     }
     if (a.nitems > 0) {
       set_tmaps(P, a, pt.shape);
@@ -775,20 +780,20 @@ int do_advance(nyx_plan *P, nyx_level *L, const double *a_old, const double *a_n
     }
   } else {
     FusedArgs a = fused_args(P, S, G, Sn, acc, predict_only);
-    if (P->prm.autotune && !P->tuned) {
+    if (untuned(P)) {
       int rc = tune_shape(P, a);
       if (rc) return rc;
     }
     // the TMA descriptors of both state versions at once (a level alternates
     // between them), so that no later step stops to build them
     prepare_tmaps(P, L);
-    if (host_out && P->ngrp > 1) {
-      for (int g = 0; g < P->ngrp; ++g) {
-        if (int rc = launch_level(P, a, g, P->stream)) return rc;
+    if (host_out && P->groups[nyx_plan::kHost].n > 1) {
+      for (int g = 0; g < P->groups[nyx_plan::kHost].n; ++g) {
+        if (int rc = launch_level(P, a, nyx_plan::kHost, g, P->stream)) return rc;
         if (int rc = read_back_group(P, Sn, g, host_out, P->stream)) return rc;
       }
     } else {
-      if (int rc = launch_level(P, a, -1, P->stream)) return rc;
+      if (int rc = launch_level(P, a, 0, -1, P->stream)) return rc;
     }
   }
   }
@@ -803,31 +808,32 @@ int do_advance(nyx_plan *P, nyx_level *L, const double *a_old, const double *a_n
   return NYX_OK;
 }
 
-// A part's items regrouped by the read-back groups [gb[g], gb[g+1]) of boxes.
-int part_groups(nyx_plan::RunPart &pt, const std::vector<int> &gb) {
+// Items regrouped by the groups [gb[g], gb[g+1]) of boxes, on the device.
+int upload_groups(const std::vector<WorkItem> &items, const std::vector<int> &gb,
+                  nyx_plan::GroupItems &v) {
   std::vector<WorkItem> it;
-  pt.grp_off.assign(1, 0);
-  group_items(pt.h_items, gb, it, pt.grp_off);
-  cudaFree(pt.d_items_grp);
-  pt.d_items_grp = nullptr;
-  CK(cudaMalloc(&pt.d_items_grp, sizeof(WorkItem) * std::max<size_t>(1, it.size())));
-  CK(cudaMemcpy(pt.d_items_grp, it.data(), sizeof(WorkItem) * it.size(), cudaMemcpyHostToDevice));
+  v.off.assign(1, 0);
+  group_items(items, gb, it, v.off);
+  CK(cudaMalloc(&v.d, sizeof(WorkItem) * std::max<size_t>(1, it.size())));
+  CK(cudaMemcpy(v.d, it.data(), sizeof(WorkItem) * it.size(), cudaMemcpyHostToDevice));
   return NYX_OK;
 }
 
-// Box groups of a fused plan, used by nyx_hydro_step_host_valid (input,
-// advance and read-back overlapped per group) and by nyx_hydro_run (each
-// group's ghost fill beside the other groups' advances): up to 32 ranges of
-// whole boxes with about equal cells (the groups' bit masks are 32 bits), as
-// long as each group keeps 2 waves of items or more in the plan's tile shape
-// (4 waves of the task form's half-size items for a run on the device, where a
-// group's tail costs more than its overlapped fill gains: 563 boxes, two
-// steps, 32.0 ms with 9 groups, 32.1 ms with 18; a run takes groups that a host
-// step made only where its own rule gives two or more).  One group (no overlap)
-// otherwise.  Every shape gets the same groups.  (On the 512^3 large level:
-// 32 groups 1.74e9 zone-updates/s end to end, 16 groups 1.72e9, 8 groups
-// 1.59e9.)
-int setup_readback(nyx_plan *P, bool host) {
+// Box groups of a fused plan for w = kHost, nyx_hydro_step_host_valid (input,
+// advance and read-back overlapped per group), or kRun, nyx_hydro_run (each
+// group's ghost fill beside the other groups' advances), made on the first such
+// call once the plan is tuned and outside a capture: up to 32 ranges of whole
+// boxes with about equal cells (the groups' bit masks are 32 bits), as long as
+// each group keeps 2 waves of items or more in the plan's tile shape (4 waves of
+// the task form's half-size items for a run on the device, where a group's tail
+// costs more than its overlapped fill gains: 563 boxes, two steps, 32.0 ms with
+// 9 groups, 32.1 ms with 18).  One group (no overlap) otherwise.  Shapes chosen
+// later take the same groups.  (On the 512^3 large level: 32 groups 1.74e9
+// zone-updates/s end to end, 16 groups 1.72e9, 8 groups 1.59e9.)
+int setup_groups(nyx_plan *P, int w) {
+  nyx_plan::BoxGroups &B = P->groups[w];
+  if (P->prm.batching == NYX_PER_BOX || B.n || untuned(P) || capturing(P)) return NYX_OK;
+  const bool host = w == nyx_plan::kHost;
   const int nsh = fused_num_shapes(P->prm.precision);
   const int grid = std::max(1, P->max_grid[P->shape]);
   int waves = P->nitems[P->shape] / grid, begun = (P->nitems[P->shape] + grid - 1) / grid;
@@ -839,12 +845,12 @@ int setup_readback(nyx_plan *P, bool host) {
       begun += (pt.nitems + pg - 1) / pg;
     }
   }
-  const int dev = fused_shape(P->shape).task ? 4 : 2, per = host ? 2 : dev;
-  P->run_groups = waves / dev > 1;
+  const int per = !host && fused_shape(P->shape).task ? 4 : 2;
   // up to four groups also where that leaves them about a wave each: the copies
-  // in and out are what is worth hiding there (27 boxes, two, three and four
-  // groups: of 64^3 6.52, 6.09 and 5.95 ms, of 48^3 3.01, 2.92 and 2.84 ms; of
-  // 32^3, 1.4 waves, one and two groups: 1.03 and 0.95 ms)
+  // in and out are what is worth hiding there (27 boxes, one, two, three and
+  // four groups: of 64^3, 5 waves, 7.35, 7.45, 6.48 and 6.29 to 6.75 ms; of 48^3
+  // 3.34, 3.41, 3.10 and 3.06 to 3.25 ms; of 32^3, 1.4 waves, two groups are
+  // taken and tie with one, 1.02 to 1.12 ms)
   const int least = host ? std::min(4, begun) : 0;
   const int G = std::min(std::min(32, P->nbox), std::max(waves / per, least));
   std::vector<int> gb(1, 0);
@@ -860,19 +866,14 @@ int setup_readback(nyx_plan *P, bool host) {
   // one group until every buffer below is in place: a set-up that fails
   // part way leaves the plan on the ungrouped path (free_plan releases what
   // was made)
-  P->ngrp = 1;
+  B.n = 1;
   if (ng < 2) return NYX_OK;
   for (int s = 0; s < nsh; ++s) {
     if (!P->d_items[s]) continue;  // not chosen yet: grouped when it is
-    std::vector<WorkItem> it;
-    P->grp_off[s].assign(1, 0);
-    group_items(P->h_items[s], gb, it, P->grp_off[s]);
-    CK(cudaMalloc(&P->d_items_grp[s], sizeof(WorkItem) * it.size()));
-    CK(cudaMemcpy(P->d_items_grp[s], it.data(), sizeof(WorkItem) * it.size(),
-                  cudaMemcpyHostToDevice));
+    if (int rc = upload_groups(P->h_items[s], gb, B.items[s])) return rc;
   }
   for (auto &pt : P->parts)
-    if (int rc = part_groups(pt, gb)) return rc;
+    if (int rc = upload_groups(pt.h_items, gb, pt.grp[w])) return rc;
   // input side: each group's fill rects, the groups they read, and an
   // input order that brings in the groups the first advances need first
   std::vector<int> gof(P->nbox);
@@ -882,19 +883,18 @@ int setup_readback(nyx_plan *P, bool host) {
   for (int p = 0; p < 4; ++p) {
     std::vector<FillRect> r;
     r.reserve(P->pass[p].h.size());
-    P->rect_off[p].assign(1, 0);
+    B.rect_off[p].assign(1, 0);
     for (int g = 0; g < ng; ++g) {
       for (const FillRect &R : P->pass[p].h) {
         if (gof[R.dst_box] != g) continue;
         r.push_back(R);
         src[g] |= 1u << gof[R.src_box];
       }
-      P->rect_off[p].push_back((int)r.size());
+      B.rect_off[p].push_back((int)r.size());
     }
     if (!r.empty()) {
-      CK(cudaMalloc(&P->d_rects_grp[p], sizeof(FillRect) * r.size()));
-      CK(cudaMemcpy(P->d_rects_grp[p], r.data(), sizeof(FillRect) * r.size(),
-                    cudaMemcpyHostToDevice));
+      CK(cudaMalloc(&B.d_rects[p], sizeof(FillRect) * r.size()));
+      CK(cudaMemcpy(B.d_rects[p], r.data(), sizeof(FillRect) * r.size(), cudaMemcpyHostToDevice));
     }
   }
   // groups advance in this order: first those whose fill reads only
@@ -915,31 +915,34 @@ int setup_readback(nyx_plan *P, bool host) {
         order.push_back(q);
       }
   }
-  CK((cudaError_t)preload_copy_kernels());
-  CK(cudaStreamCreateWithFlags(&P->copy_stream, cudaStreamNonBlocking));
-  CK(cudaStreamCreateWithFlags(&P->h2d_stream, cudaStreamNonBlocking));
-  CK(cudaStreamCreateWithFlags(&P->stream2, cudaStreamNonBlocking));
-  CK(cudaEventCreateWithFlags(&P->ev_start, cudaEventDisableTiming));
-  CK(cudaEventCreateWithFlags(&P->ev_setup, cudaEventDisableTiming));
-  CK(cudaEventCreateWithFlags(&P->ev_side, cudaEventDisableTiming));
-  CK(cudaMalloc(&P->d_queue_grp, sizeof(int) * ng));
-  P->ev_grp.assign(ng, nullptr);
-  for (auto &e : P->ev_grp) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  P->ev_in.assign(ng, nullptr);
-  for (auto &e : P->ev_in) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  for (int k = 0; k < 2; ++k) {
-    CK(cudaStreamCreateWithFlags(&P->fill_stream[k], cudaStreamNonBlocking));
-    CK(cudaEventCreateWithFlags(&P->ev_fjoin[k], cudaEventDisableTiming));
+  const auto stream = [](cudaStream_t *q) {
+    return *q ? cudaSuccess : cudaStreamCreateWithFlags(q, cudaStreamNonBlocking);
+  };
+  const auto event = [](cudaEvent_t *q) {
+    return *q ? cudaSuccess : cudaEventCreateWithFlags(q, cudaEventDisableTiming);
+  };
+  if (host) {
+    CK((cudaError_t)preload_copy_kernels());
+    CK(stream(&P->copy_stream));
+    CK(stream(&P->h2d_stream));
+  } else {
+    for (int k = 0; k < 2; ++k) {
+      CK(stream(&P->fill_stream[k]));
+      CK(event(&P->ev_fjoin[k]));
+    }
   }
-  P->ev_gfill.assign(ng, nullptr);
-  for (auto &e : P->ev_gfill) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  P->ev_gadv.assign(ng, nullptr);
-  for (auto &e : P->ev_gadv) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  P->grp_src = src;
-  P->in_order = order;
-  P->proc_order = proc;
-  P->grp_box = gb;
-  P->ngrp = ng;
+  CK(stream(&P->stream2));
+  for (cudaEvent_t *q : {&P->ev_start, &P->ev_setup, &P->ev_side}) CK(event(q));
+  CK(cudaMalloc(&B.d_queue, sizeof(int) * ng));
+  for (auto *v : {&B.ev_ready, &B.ev_done}) {
+    v->assign(ng, nullptr);
+    for (auto &e : *v) CK(event(&e));
+  }
+  B.src = src;
+  B.in_order = order;
+  B.proc_order = proc;
+  B.box = gb;
+  B.n = ng;
   return NYX_OK;
 }
 
@@ -952,10 +955,11 @@ int setup_readback(nyx_plan *P, bool host) {
 int step_pipelined(nyx_plan *P, nyx_level *L, const double *host_in, double *host_out) {
   double *S = L->state[L->cur];
   double *Sn = L->state[1 - L->cur];
+  const nyx_plan::BoxGroups &B = P->groups[nyx_plan::kHost];
   CK(cudaEventRecord(P->ev_start, P->stream));
   CK(cudaStreamWaitEvent(P->h2d_stream, P->ev_start, 0));
-  for (int q : P->in_order) {
-    const int b0 = P->grp_box[q], b1 = P->grp_box[q + 1];
+  for (int q : B.in_order) {
+    const int b0 = B.box[q], b1 = B.box[q + 1];
     const long long c0 = P->cell_pref[b0], c1 = b1 < P->nbox ? P->cell_pref[b1] : P->total_cells;
     const int k0 = P->plane_pref[b0], k1 = b1 < P->nbox ? P->plane_pref[b1] : P->plane_blocks;
     CK(cudaMemcpyAsync(P->d_packed + NCONS * c0, host_in + NCONS * c0,
@@ -964,7 +968,7 @@ int step_pipelined(nyx_plan *P, nyx_level *L, const double *host_in, double *hos
     launch_valid_copy(S, P->d_packed, P->d_boxes, P->d_cell_pref, P->d_plane_pref, P->nbox,
                       k1 - k0, k0, 1, P->h2d_stream);
     P->launches += 1;
-    CK(cudaEventRecord(P->ev_in[q], P->h2d_stream));
+    CK(cudaEventRecord(B.ev_ready[q], P->h2d_stream));
   }
   launch_step_setup(P->d_K, P->d_scal, P->d_scal + 1, P->d_scal + 2, P->d_SC, P->d_boxes, P->nbox,
                     P->d_BS, P->stream);
@@ -974,24 +978,24 @@ int step_pipelined(nyx_plan *P, nyx_level *L, const double *host_in, double *hos
   FusedArgs a = fused_args(P, S, L->grav, Sn, P->d_dtacc, false);
   const cudaStream_t cs[2] = {P->stream, P->stream2};
   unsigned waited[2] = {0u, 0u};
-  for (int gi = 0; gi < P->ngrp; ++gi) {
-    const int g = P->proc_order[gi];
+  for (int gi = 0; gi < B.n; ++gi) {
+    const int g = B.proc_order[gi];
     const cudaStream_t st = cs[gi & 1];
-    const unsigned need = (P->grp_src[g] | (1u << g)) & ~waited[gi & 1];
-    for (int q = 0; q < P->ngrp; ++q)
-      if ((need >> q) & 1u) CK(cudaStreamWaitEvent(st, P->ev_in[q], 0));
+    const unsigned need = (B.src[g] | (1u << g)) & ~waited[gi & 1];
+    for (int q = 0; q < B.n; ++q)
+      if ((need >> q) & 1u) CK(cudaStreamWaitEvent(st, B.ev_ready[q], 0));
     waited[gi & 1] |= need;
     for (int p = 0; p < 4; ++p) {
-      const int r0 = P->rect_off[p][g], nr = P->rect_off[p][g + 1] - r0;
+      const int r0 = B.rect_off[p][g], nr = B.rect_off[p][g + 1] - r0;
       if (nr > 0) {
-        launch_fill(S, NCONS, P->d_boxes, P->d_rects_grp[p] + r0, nullptr, nr, P->pass[p].total,
+        launch_fill(S, NCONS, P->d_boxes, B.d_rects[p] + r0, nullptr, nr, P->pass[p].total,
                     st, true);
         P->launches += 1;
       }
     }
     if (P->d_flat) {
       // the group's flattening coefficients read only its own boxes, ghosts included
-      const int t0 = P->flat_tile_pref[P->grp_box[g]], t1 = P->flat_tile_pref[P->grp_box[g + 1]];
+      const int t0 = P->flat_tile_pref[B.box[g]], t1 = P->flat_tile_pref[B.box[g + 1]];
       if (t1 > t0) {
         int e = launch_flatten(P->prm.precision, P->d_boxes, P->d_flat_tiles + t0, t1 - t0, S,
                                P->d_K, P->d_flat, st);
@@ -999,8 +1003,8 @@ int step_pipelined(nyx_plan *P, nyx_level *L, const double *host_in, double *hos
         P->launches += 1;
       }
     }
-    a.queue = P->d_queue_grp + g;
-    if (int rc = launch_level(P, a, g, st)) return rc;
+    a.queue = B.d_queue + g;
+    if (int rc = launch_level(P, a, nyx_plan::kHost, g, st)) return rc;
     if (int rc = read_back_group(P, Sn, g, host_out, st)) return rc;
   }
   CK(cudaEventRecord(P->ev_side, P->stream2));
@@ -1018,14 +1022,15 @@ int step_pipelined(nyx_plan *P, nyx_level *L, const double *host_in, double *hos
 // on stream st (where the group advanced), then copied to host_out on the
 // copy stream.
 int read_back_group(nyx_plan *P, const double *Sn, int g, double *host_out, cudaStream_t st) {
-  const int b0 = P->grp_box[g], b1 = P->grp_box[g + 1];
+  const nyx_plan::BoxGroups &B = P->groups[nyx_plan::kHost];
+  const int b0 = B.box[g], b1 = B.box[g + 1];
   const int k0 = P->plane_pref[b0], k1 = b1 < P->nbox ? P->plane_pref[b1] : P->plane_blocks;
   launch_valid_copy(const_cast<double *>(Sn), P->d_packed, P->d_boxes, P->d_cell_pref,
                     P->d_plane_pref, P->nbox, k1 - k0, k0, 0, st);
   P->launches += 1;
   const long long c0 = P->cell_pref[b0], c1 = b1 < P->nbox ? P->cell_pref[b1] : P->total_cells;
-  CK(cudaEventRecord(P->ev_grp[g], st));
-  CK(cudaStreamWaitEvent(P->copy_stream, P->ev_grp[g], 0));
+  CK(cudaEventRecord(B.ev_done[g], st));
+  CK(cudaStreamWaitEvent(P->copy_stream, B.ev_done[g], 0));
   CK(cudaMemcpyAsync(host_out + NCONS * c0, P->d_packed + NCONS * c0,
                      sizeof(double) * NCONS * (size_t)(c1 - c0), cudaMemcpyDeviceToHost,
                      P->copy_stream));
@@ -1284,8 +1289,11 @@ int tune_shape(nyx_plan *P, const FusedArgs &base) {
     CK(cudaMemcpy(pt.d_items, pt.h_items.data(), sizeof(WorkItem) * pt.nitems,
                   cudaMemcpyHostToDevice));
     P->parts.push_back(std::move(pt));
-    if (P->ngrp > 1)
-      if (int r2 = part_groups(P->parts.back(), P->grp_box)) return r2;
+    for (int w = 0; w < 2; ++w)
+      if (P->groups[w].n > 1)
+        if (int r2 = upload_groups(P->parts.back().h_items, P->groups[w].box,
+                                   P->parts.back().grp[w]))
+          return r2;
   }
   return NYX_OK;
 }
@@ -1307,29 +1315,30 @@ int tune_shape(nyx_plan *P, const FusedArgs &base) {
 // Every cell takes the same arithmetic as in the one-launch form, so the
 // result is the same bit for bit.
 int run_grouped(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev, int nsteps) {
+  const nyx_plan::BoxGroups &B = P->groups[nyx_plan::kRun];
   CK(cudaEventRecord(P->ev_start, P->stream));
   for (int k = 0; k < 2; ++k) CK(cudaStreamWaitEvent(P->fill_stream[k], P->ev_start, 0));
   const cudaStream_t cs[2] = {P->stream, P->stream2};
   for (int s = 0; s < nsteps; ++s) {
     double *S = L->state[L->cur];
     double *Sn = L->state[1 - L->cur];
-    for (int gi = 0; gi < P->ngrp; ++gi) {
-      const int g = P->proc_order[gi];
+    for (int gi = 0; gi < B.n; ++gi) {
+      const int g = B.proc_order[gi];
       const cudaStream_t fs = P->fill_stream[gi & 1];
       if (s > 0) {
-        const unsigned need = P->grp_src[g] | (1u << g);
-        for (int q = 0; q < P->ngrp; ++q)
-          if ((need >> q) & 1u) CK(cudaStreamWaitEvent(fs, P->ev_gadv[q], 0));
+        const unsigned need = B.src[g] | (1u << g);
+        for (int q = 0; q < B.n; ++q)
+          if ((need >> q) & 1u) CK(cudaStreamWaitEvent(fs, B.ev_done[q], 0));
       }
       for (int p = 0; p < 4; ++p) {
-        const int r0 = P->rect_off[p][g], nr = P->rect_off[p][g + 1] - r0;
+        const int r0 = B.rect_off[p][g], nr = B.rect_off[p][g + 1] - r0;
         if (nr > 0) {
-          launch_fill(S, NCONS, P->d_boxes, P->d_rects_grp[p] + r0, nullptr, nr,
+          launch_fill(S, NCONS, P->d_boxes, B.d_rects[p] + r0, nullptr, nr,
                       P->pass[p].total, fs, true);
           P->launches += 1;
         }
       }
-      CK(cudaEventRecord(P->ev_gfill[g], fs));
+      CK(cudaEventRecord(B.ev_ready[g], fs));
     }
     if (P->d_flat) {
       // the coefficient pass (512 threads, 43 KB of shared memory per block)
@@ -1347,13 +1356,13 @@ int run_grouped(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev, 
     CK(cudaEventRecord(P->ev_setup, P->stream));
     CK(cudaStreamWaitEvent(P->stream2, P->ev_setup, 0));
     FusedArgs a = fused_args(P, S, L->grav, Sn, P->d_dtacc, false);
-    for (int gi = 0; gi < P->ngrp; ++gi) {
-      const int g = P->proc_order[gi];
+    for (int gi = 0; gi < B.n; ++gi) {
+      const int g = B.proc_order[gi];
       const cudaStream_t st = cs[gi & 1];
-      CK(cudaStreamWaitEvent(st, P->ev_gfill[g], 0));
-      a.queue = P->d_queue_grp + g;
-      if (int rc = launch_level(P, a, g, st)) return rc;
-      CK(cudaEventRecord(P->ev_gadv[g], st));
+      CK(cudaStreamWaitEvent(st, B.ev_ready[g], 0));
+      a.queue = B.d_queue + g;
+      if (int rc = launch_level(P, a, nyx_plan::kRun, g, st)) return rc;
+      CK(cudaEventRecord(B.ev_done[g], st));
     }
     CK(cudaEventRecord(P->ev_side, P->stream2));
     CK(cudaStreamWaitEvent(P->stream, P->ev_side, 0));
@@ -1378,8 +1387,8 @@ int enqueue_run(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev, 
   // fused plans with box groups overlap each step's ghost fill with the
   // advance; profiled runs keep one fill and one advance launch per step so
   // that each is timed on its own
-  if (P->prm.batching != NYX_PER_BOX && P->ngrp > 1 && !(P->prm.autotune && !P->tuned) &&
-      !P->profiling && P->run_groups && nsteps > 0) {
+  if (P->prm.batching != NYX_PER_BOX && P->groups[nyx_plan::kRun].n > 1 && !P->profiling &&
+      nsteps > 0) {
     prepare_tmaps(P, L);
     return run_grouped(P, L, a_dev, dt_dev, nsteps);
   }
@@ -1784,12 +1793,11 @@ int nyx_hydro_run(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev
   if (!P || !L || !a_dev || !dt_dev || nsteps < 0) return fail(NYX_EINVAL, "null argument");
   if ((L->cur != 0 && L->cur != 1) || !L->state[0] || !L->state[1] || L->state[0] == L->state[1])
     return fail(NYX_EINVAL, "level needs two distinct state buffers and cur in {0,1}");
-  // box groups (made once, outside any capture): a run overlaps each group's
-  // ghost fill with the other groups' advances
-  if (P->prm.batching != NYX_PER_BOX && P->ngrp == 0)
-    if (int rc = setup_readback(P, false)) return rc;
-  if (!use_graph) return enqueue_run(P, L, a_dev, dt_dev, nsteps, compute_dt0);
-  if (P->prm.batching == NYX_PERSISTENT && P->prm.autotune && !P->tuned) {
+  if (!use_graph) {
+    if (int rc = setup_groups(P, nyx_plan::kRun)) return rc;
+    return enqueue_run(P, L, a_dev, dt_dev, nsteps, compute_dt0);
+  }
+  if (P->prm.batching == NYX_PERSISTENT && untuned(P)) {
     // tune outside the capture: one eager step on scratch copies is not
     // possible without the caller's buffers, so tune on the real ones and
     // redo the work below (the tuning launches only write state[1-cur]).
@@ -1814,6 +1822,7 @@ int nyx_hydro_run(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev
     int rc = tune_shape(P, a);
     if (rc) return rc;
   }
+  if (int rc = setup_groups(P, nyx_plan::kRun)) return rc;
   if (P->prm.batching == NYX_PERSISTENT) prepare_tmaps(P, L);
   if (P->graphs_gen != P->shape_gen) {  // recorded with another shape
     CK(cudaStreamSynchronize(P->stream));
@@ -1912,13 +1921,13 @@ int nyx_hydro_step_host_valid(nyx_plan *P, nyx_level *L, const double *host_in, 
     P->plane_blocks = (int)nb;
     P->plane_pref = pp;
   }
-  if (P->prm.batching != NYX_PER_BOX && P->ngrp == 0)
-    if (int rc = setup_readback(P, true)) return rc;
-  if (P->prm.batching != NYX_PER_BOX && !(P->prm.autotune && !P->tuned)) prepare_tmaps(P, L);
+  if (int rc = setup_groups(P, nyx_plan::kHost)) return rc;
+  const bool grouped = P->groups[nyx_plan::kHost].n > 1;
+  if (P->prm.batching != NYX_PER_BOX && !untuned(P)) prepare_tmaps(P, L);
   const size_t bytes = sizeof(double) * NCONS * (size_t)P->total_cells;
   double h[3] = {a_old, a_new, *dt_inout};
   CK(cudaMemcpyAsync(P->d_scal, h, 3 * sizeof(double), cudaMemcpyHostToDevice, P->stream));
-  if (P->ngrp > 1 && *dt_inout > 0.0 && !(P->prm.autotune && !P->tuned)) {
+  if (grouped && *dt_inout > 0.0) {
     // input, advance and read-back overlapped per box group
     int rc = step_pipelined(P, L, host_in, host_out);
     if (rc) {
@@ -1940,7 +1949,7 @@ int nyx_hydro_step_host_valid(nyx_plan *P, nyx_level *L, const double *host_in, 
                     P->nbox, P->plane_blocks, 0, 1, P->stream);
   P->launches += 1;
   if (!(*dt_inout > 0.0)) do_estdt(P, L->state[L->cur], P->d_scal, P->d_scal + 2);
-  if (P->ngrp > 1) {
+  if (grouped) {
     // the read-back of each box group overlaps the advance of the next ones
     int rc = do_advance(P, L, P->d_scal, P->d_scal + 1, P->d_scal + 2, nullptr, P->d_scal + 3,
                         false, host_out);

@@ -73,41 +73,42 @@ struct nyx_plan {
   int *d_plane_pref = nullptr;
   std::vector<int> plane_pref;
   int plane_blocks = 0;
-  // ... and its read-back overlapped with the advance: the fused form's
-  // items regrouped by box ranges [grp_box[g], grp_box[g+1]) (each group in
-  // queue order), one launch per group; a group's cells are gathered and
-  // copied to the host on copy_stream while the next group advances
-  int ngrp = 0;
-  bool run_groups = false;  // also used by runs on the device
-  std::vector<int> grp_box;
-  std::vector<int> grp_off[8];  // per shape: first item of each group, ngrp + 1 entries
-  nyx::WorkItem *d_items_grp[8] = {nullptr};
-  cudaStream_t copy_stream = nullptr;
-  std::vector<cudaEvent_t> ev_grp;
-  // ... and its input overlapped too: each group's cells copied in and
-  // scattered on h2d_stream (in in_order), each group's ghost fill (the
-  // rects of pass p whose destination is in group g: d_rects_grp[p] from
-  // rect_off[p][g]) launched once the groups it reads (grp_src[g], a bit
-  // mask) are in
-  cudaStream_t h2d_stream = nullptr;
-  std::vector<cudaEvent_t> ev_in;
-  cudaEvent_t ev_start = nullptr;
-  // groups advance on the plan's stream and stream2 in turn (a group's
-  // launch takes the SMs its predecessor's tail frees), each with its own
-  // work-queue counter
-  cudaStream_t stream2 = nullptr;
-  cudaEvent_t ev_setup = nullptr, ev_side = nullptr;
-  int *d_queue_grp = nullptr;
-  nyx::FillRect *d_rects_grp[4] = {nullptr};
-  std::vector<int> rect_off[4];
-  std::vector<unsigned> grp_src;
-  std::vector<int> in_order;
-  std::vector<int> proc_order;  // the order in which the groups advance
-  // multi-step runs on the device (nyx_hydro_run): each group's ghost fill
-  // of step s+1 runs on one of two fill streams as soon as the groups it
-  // reads have advanced in step s, beside the other groups' advances
+  // Box groups: the fused form's items regrouped by box ranges [box[g],
+  // box[g+1]) (each group in queue order), one launch per group.  Host steps
+  // (nyx_hydro_step_host_valid) and runs on the device (nyx_hydro_run) weigh
+  // different things, so each has its own, made on first use.
+  struct GroupItems {
+    nyx::WorkItem *d = nullptr;
+    std::vector<int> off;  // first item of each group, n + 1 entries
+  };
+  struct BoxGroups {
+    int n = 0;  // 0: not made yet, 1: no grouping
+    std::vector<int> box;
+    GroupItems items[8];  // per shape
+    // ghost fill of group g: the rects of pass p whose destination is in g,
+    // d_rects[p] from rect_off[p][g]; it reads the groups of the bit mask src[g]
+    nyx::FillRect *d_rects[4] = {nullptr};
+    std::vector<int> rect_off[4];
+    std::vector<unsigned> src;
+    std::vector<int> in_order;    // host steps: the order of the inputs
+    std::vector<int> proc_order;  // the order in which the groups advance
+    int *d_queue = nullptr;       // a work-queue counter per group
+    // host steps: group g's cells are in, and gathered for the way back;
+    // runs: group g's ghost cells are filled, and it has advanced
+    std::vector<cudaEvent_t> ev_ready, ev_done;
+  };
+  enum { kHost, kRun };
+  BoxGroups groups[2];
+  // streams and events of both.  Host steps: each group's cells are copied in
+  // and scattered on h2d_stream (in in_order), and its new cells gathered and
+  // copied to the host on copy_stream while the next group advances.  Groups
+  // advance on the plan's stream and stream2 in turn (a group's launch takes
+  // the SMs its predecessor's tail frees).  Runs: each group's ghost fill of
+  // step s+1 runs on one of two fill streams as soon as the groups it reads
+  // have advanced in step s, beside the other groups' advances.
+  cudaStream_t copy_stream = nullptr, h2d_stream = nullptr, stream2 = nullptr;
   cudaStream_t fill_stream[2] = {nullptr, nullptr};
-  std::vector<cudaEvent_t> ev_gfill, ev_gadv;
+  cudaEvent_t ev_start = nullptr, ev_setup = nullptr, ev_side = nullptr;
   cudaEvent_t ev_fjoin[2] = {nullptr, nullptr};
   // per-box FP64 form
   double *d_scratch = nullptr;
@@ -126,8 +127,7 @@ struct nyx_plan {
     nyx::WorkItem *d_items = nullptr;
     int nitems = 0;
     std::vector<nyx::WorkItem> h_items;
-    nyx::WorkItem *d_items_grp = nullptr;
-    std::vector<int> grp_off;  // first item of each read-back group, ngrp + 1 entries
+    GroupItems grp[2];  // regrouped for host steps and for runs
   };
   std::vector<RunPart> parts;
   // parts given up for another shape: graphs recorded earlier, the plan's own

@@ -1,5 +1,6 @@
-"""What an earlier call leaves in a plan does not change a later one: tile
-shapes changed between replays of a run's graph."""
+"""What an earlier call leaves in a plan does not change a later one: box
+groups made by a run and by a host step, tile shapes changed between replays
+of a run's graph."""
 import numpy as np
 import pytest
 
@@ -21,6 +22,51 @@ def _plan(w, **kw):
     return H.Plan(w.level, gamma=w.gamma, cfl=w.cfl, precision="mixed", **kw)
 
 
+def _run(plan, w, **kw):
+    """One step from the workload's state: (launches, new valid cells)."""
+    lev = H.make_level(plan, w.state, w.grav)
+    a, d = _scalars()
+    plan.counters(reset=True)
+    plan.run(lev, a, d, 1, compute_dt0=True, use_graph=False)
+    torch.cuda.synchronize()
+    assert plan.status()[0] == H.NYX_OK
+    return plan.counters(reset=True)["launches"], [W.valid(x) for x in
+                                                   plan.from_device(lev.current, 6)]
+
+
+def _host(plan, w, dt):
+    """One overlapped host step: (launches, new valid cells)."""
+    lev = H.make_level(plan, w.state, w.grav)
+    h_in = torch.from_numpy(plan.pack_valid(w.state)).pin_memory()
+    h_out = torch.empty_like(h_in).pin_memory()
+    plan.counters(reset=True)
+    plan.step_host_valid(lev, h_in, h_out, A[0], A[1], dt)
+    assert plan.status()[0] == H.NYX_OK
+    return plan.counters(reset=True)["launches"], plan.unpack_valid(h_out.numpy())
+
+
+# 27 boxes of 32^3 (1.4 waves: host steps overlap, runs do not) and 1000 boxes
+# of 16^3 (13 waves: both do, by rules of their own)
+@pytest.mark.parametrize("n,box", [(96, 32), (160, 16)])
+def test_host_steps_and_runs_group_the_boxes_in_either_order(n, box):
+    w = W.tiled_box(n=n, box=box, nsteps=1)
+    dt = 1e-5
+    p, q = _plan(w), _plan(w)
+    host_first, s0 = _host(p, w, dt)
+    run_after, s1 = _run(p, w)
+    run_first, s2 = _run(q, w)
+    host_after, s3 = _host(q, w, dt)
+    assert host_after == host_first and run_after == run_first
+    # a host step's group adds a gather and an advance launch to the run's
+    assert host_first > run_first
+    for x, y in zip(s0, s3):
+        assert np.array_equal(x, y)
+    for x, y in zip(s1, s2):
+        assert np.array_equal(x, y)
+    p.close()
+    q.close()
+
+
 def _cache(monkeypatch, tmp_path, **picks):
     """A tuning cache that answers extent -> (shape, CTAs per SM)."""
     props = torch.cuda.get_device_properties(0)
@@ -30,6 +76,26 @@ def _cache(monkeypatch, tmp_path, **picks):
         f' "{prefix}{e[1:]}": {{"shape": {s}, "ctas_per_sm": {c}, "ns_per_zone": 1}}'
         for e, (s, c) in picks.items()) + "\n}\n")
     monkeypatch.setenv("NYX_TUNE_CACHE", str(f))
+
+
+def test_a_run_groups_the_boxes_by_the_tuned_shape(tmp_path, monkeypatch):
+    # 8 x 8 tiles at one CTA per SM: 26 waves, 6 groups; the shape before
+    # tuning has 13 waves, 3 groups
+    _cache(monkeypatch, tmp_path, x16x16x16=(4, 1))
+    w = W.tiled_box(n=160, box=16, nsteps=1)
+    p, q = _plan(w, autotune=1), _plan(w, autotune=1)
+    _run(p, w)                       # tunes
+    lev = H.make_level(q, w.state, w.grav)
+    a, d = _scalars(1e-5)
+    q.advance(lev, a[:1], a[1:2], d[:1])  # tunes too, without groups
+    assert p.tune_info() == q.tune_info() and p.tune_info()[2] == 1
+    n_p, s_p = _run(p, w)
+    n_q, s_q = _run(q, w)
+    assert n_p == n_q
+    for x, y in zip(s_p, s_q):
+        assert np.array_equal(x, y)
+    p.close()
+    q.close()
 
 
 class _Graphed:
