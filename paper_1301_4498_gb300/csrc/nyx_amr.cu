@@ -305,14 +305,14 @@ void free_amr(nyx_amr *A) {
 }
 
 template <class T>
-int upload(const std::vector<T> &h, T **d) {
+int upload(const nyx_plan *P, const std::vector<T> &h, T **d) {
   *d = nullptr;
   if (h.empty()) return NYX_OK;
   cudaError_t e = cudaMalloc(d, sizeof(T) * h.size());
   if (e != cudaSuccess)
     return e == cudaErrorMemoryAllocation ? fail(NYX_ENOMEM, "amr table allocation failed")
                                           : cuda_fail(e, "cudaMalloc");
-  CK(cudaMemcpy(*d, h.data(), sizeof(T) * h.size(), cudaMemcpyHostToDevice));
+  CK(plan_upload(P, *d, h.data(), sizeof(T) * h.size()));
   return NYX_OK;
 }
 
@@ -583,17 +583,17 @@ int build_tables(nyx_amr *A) {
   for (const AvgRect &R : avg) split_avg(R, avg2);
   avg.swap(avg2);
   int rc;
-  if ((rc = upload(ig, &A->d_ig))) return rc;
-  if ((rc = upload(ia, &A->d_ia))) return rc;
+  if ((rc = upload(A->C, ig, &A->d_ig))) return rc;
+  if ((rc = upload(A->C, ia, &A->d_ia))) return rc;
   A->n_ig = (int)ig.size();
   A->n_ia = (int)ia.size();
   for (int o = 0; o < 6; ++o) {
-    if ((rc = upload(face[o], &A->d_face[o]))) return rc;
+    if ((rc = upload(A->C, face[o], &A->d_face[o]))) return rc;
     A->n_face[o] = (int)face[o].size();
   }
-  if ((rc = upload(avg, &A->d_avg))) return rc;
+  if ((rc = upload(A->C, avg, &A->d_avg))) return rc;
   A->n_avg = (int)avg.size();
-  if ((rc = upload(cov, &A->d_cov))) return rc;
+  if ((rc = upload(A->C, cov, &A->d_cov))) return rc;
   return NYX_OK;
 }
 

@@ -248,7 +248,7 @@ std::vector<FillRect> cut_rects(const std::vector<FillRect> &rects) {
   return out;
 }
 
-int upload_pass(FillPass &p, const std::vector<FillRect> &whole) {
+int upload_pass(const nyx_plan *P, FillPass &p, const std::vector<FillRect> &whole) {
   const std::vector<FillRect> rects = cut_rects(whole);
   p.n = (int)rects.size();
   if (!p.n) return NYX_OK;
@@ -262,8 +262,8 @@ int upload_pass(FillPass &p, const std::vector<FillRect> &whole) {
   p.h = rects;
   CK(cudaMalloc(&p.d_rects, sizeof(FillRect) * p.n));
   CK(cudaMalloc(&p.d_pref, sizeof(long long) * p.n));
-  CK(cudaMemcpy(p.d_rects, rects.data(), sizeof(FillRect) * p.n, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(p.d_pref, pref.data(), sizeof(long long) * p.n, cudaMemcpyHostToDevice));
+  CK(plan_upload(P, p.d_rects, rects.data(), sizeof(FillRect) * p.n));
+  CK(plan_upload(P, p.d_pref, pref.data(), sizeof(long long) * p.n));
   return NYX_OK;
 }
 
@@ -421,7 +421,7 @@ void group_items(const std::vector<WorkItem> &items, const std::vector<int> &gb,
 // creation, nyx_hydro_set_tile_shape, the autotuner): a plan runs one shape,
 // and simulating the queues of all of them took most of a plan's set-up.
 // Relaxed capture mode: the allocation and the upload touch no stream that a
-// caller may be capturing.
+// caller may be capturing (plan_upload has its own).
 int ensure_items(nyx_plan *P, int s) {
   if (P->d_items[s]) return NYX_OK;
   std::vector<std::array<int, 3>> n(P->nbox);
@@ -434,7 +434,7 @@ int ensure_items(nyx_plan *P, int s) {
   auto upload = [&](const std::vector<WorkItem> &v, WorkItem **d) {
     cudaError_t e = cudaMalloc(d, sizeof(WorkItem) * std::max<size_t>(1, v.size()));
     if (e != cudaSuccess) return e;
-    e = cudaMemcpy(*d, v.data(), sizeof(WorkItem) * v.size(), cudaMemcpyHostToDevice);
+    e = plan_upload(P, *d, v.data(), sizeof(WorkItem) * v.size());
     if (e != cudaSuccess) {
       cudaFree(*d);
       *d = nullptr;
@@ -520,6 +520,7 @@ void free_plan(nyx_plan *P) {
     if (P->ev_fjoin[k]) cudaEventDestroy(P->ev_fjoin[k]);
   }
   cudaFree(P->d_queue);
+  if (P->up_stream) cudaStreamDestroy(P->up_stream);
   delete P;
 }
 
@@ -674,8 +675,7 @@ const void *plan_tmaps(nyx_plan *P, const double *field, int ncomp, int shape) {
                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     }
     if (ok && cudaMalloc(&d, sizeof(CUtensorMap) * h.size()) == cudaSuccess) {
-      if (cudaMemcpy(d, h.data(), sizeof(CUtensorMap) * h.size(), cudaMemcpyHostToDevice) !=
-          cudaSuccess) {
+      if (plan_upload(P, d, h.data(), sizeof(CUtensorMap) * h.size()) != cudaSuccess) {
         cudaFree(d);
         d = nullptr;
       }
@@ -809,13 +809,13 @@ int do_advance(nyx_plan *P, nyx_level *L, const double *a_old, const double *a_n
 }
 
 // Items regrouped by the groups [gb[g], gb[g+1]) of boxes, on the device.
-int upload_groups(const std::vector<WorkItem> &items, const std::vector<int> &gb,
-                  nyx_plan::GroupItems &v) {
+int upload_groups(const nyx_plan *P, const std::vector<WorkItem> &items,
+                  const std::vector<int> &gb, nyx_plan::GroupItems &v) {
   std::vector<WorkItem> it;
   v.off.assign(1, 0);
   group_items(items, gb, it, v.off);
   CK(cudaMalloc(&v.d, sizeof(WorkItem) * std::max<size_t>(1, it.size())));
-  CK(cudaMemcpy(v.d, it.data(), sizeof(WorkItem) * it.size(), cudaMemcpyHostToDevice));
+  CK(plan_upload(P, v.d, it.data(), sizeof(WorkItem) * it.size()));
   return NYX_OK;
 }
 
@@ -870,10 +870,10 @@ int setup_groups(nyx_plan *P, int w) {
   if (ng < 2) return NYX_OK;
   for (int s = 0; s < nsh; ++s) {
     if (!P->d_items[s]) continue;  // not chosen yet: grouped when it is
-    if (int rc = upload_groups(P->h_items[s], gb, B.items[s])) return rc;
+    if (int rc = upload_groups(P, P->h_items[s], gb, B.items[s])) return rc;
   }
   for (auto &pt : P->parts)
-    if (int rc = upload_groups(pt.h_items, gb, pt.grp[w])) return rc;
+    if (int rc = upload_groups(P, pt.h_items, gb, pt.grp[w])) return rc;
   // input side: each group's fill rects, the groups they read, and an
   // input order that brings in the groups the first advances need first
   std::vector<int> gof(P->nbox);
@@ -894,7 +894,7 @@ int setup_groups(nyx_plan *P, int w) {
     }
     if (!r.empty()) {
       CK(cudaMalloc(&B.d_rects[p], sizeof(FillRect) * r.size()));
-      CK(cudaMemcpy(B.d_rects[p], r.data(), sizeof(FillRect) * r.size(), cudaMemcpyHostToDevice));
+      CK(plan_upload(P, B.d_rects[p], r.data(), sizeof(FillRect) * r.size()));
     }
   }
   // groups advance in this order: first those whose fill reads only
@@ -1226,7 +1226,7 @@ int tune_shape(nyx_plan *P, const FusedArgs &base) {
           }
           wave_cap = wave.size();
         }
-        CK(cudaMemcpy(d_wave, wave.data(), sizeof(WorkItem) * wave.size(), cudaMemcpyHostToDevice));
+        CK(plan_upload(P, d_wave, wave.data(), sizeof(WorkItem) * wave.size()));
         FusedArgs a = base;
         a.items = d_wave;
         a.nitems = 2 * grid;
@@ -1286,12 +1286,11 @@ int tune_shape(nyx_plan *P, const FusedArgs &base) {
     pt.h_items = subset_items(*P, kv.second, ts.tx, ts.ty, pt.grid, P->prm.z_chunks != 0, !ts.task);
     pt.nitems = (int)pt.h_items.size();
     CK(cudaMalloc(&pt.d_items, sizeof(WorkItem) * std::max(1, pt.nitems)));
-    CK(cudaMemcpy(pt.d_items, pt.h_items.data(), sizeof(WorkItem) * pt.nitems,
-                  cudaMemcpyHostToDevice));
+    CK(plan_upload(P, pt.d_items, pt.h_items.data(), sizeof(WorkItem) * pt.nitems));
     P->parts.push_back(std::move(pt));
     for (int w = 0; w < 2; ++w)
       if (P->groups[w].n > 1)
-        if (int r2 = upload_groups(P->parts.back().h_items, P->groups[w].box,
+        if (int r2 = upload_groups(P, P->parts.back().h_items, P->groups[w].box,
                                    P->parts.back().grp[w]))
           return r2;
   }
@@ -1403,6 +1402,13 @@ int enqueue_run(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev, 
 
 namespace nyx {
 namespace host {
+
+cudaError_t plan_upload(const nyx_plan *P, void *dst, const void *src, size_t bytes) {
+  const cudaError_t e =
+      src ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, P->up_stream)
+          : cudaMemsetAsync(dst, 0, bytes, P->up_stream);
+  return e == cudaSuccess ? cudaStreamSynchronize(P->up_stream) : e;
+}
 
 int plan_fill(nyx_plan *P, double *field, int ncomp) { return do_fill(P, field, ncomp); }
 
@@ -1611,12 +1617,12 @@ int nyx_hydro_plan(const nyx_level_desc *lev, const nyx_hydro_params *prm, void 
     }                                                            \
   } while (0)
   {
-    for (int p = 0; p < 4; ++p) TRY(upload_pass(P->pass[p], rects[p]));
+    TRYC(cudaStreamCreateWithFlags(&P->up_stream, cudaStreamNonBlocking));
+    for (int p = 0; p < 4; ++p) TRY(upload_pass(P, P->pass[p], rects[p]));
     TRYC(cudaMalloc(&P->d_boxes, sizeof(BoxDev) * P->nbox));
-    TRYC(cudaMemcpy(P->d_boxes, P->hbox.data(), sizeof(BoxDev) * P->nbox, cudaMemcpyHostToDevice));
+    TRYC(plan_upload(P, P->d_boxes, P->hbox.data(), sizeof(BoxDev) * P->nbox));
     TRYC(cudaMalloc(&P->d_cell_pref, sizeof(long long) * P->nbox));
-    TRYC(cudaMemcpy(P->d_cell_pref, P->cell_pref.data(), sizeof(long long) * P->nbox,
-                    cudaMemcpyHostToDevice));
+    TRYC(plan_upload(P, P->d_cell_pref, P->cell_pref.data(), sizeof(long long) * P->nbox));
     SchemeConsts &K = P->hK;
     K.gamma = prm->gamma;
     K.gm1 = prm->gamma - 1.0;
@@ -1637,16 +1643,16 @@ int nyx_hydro_plan(const nyx_level_desc *lev, const nyx_hydro_params *prm, void 
     K.linear_rs = prm->riemann_solver == NYX_RS_LINEAR;
     K.flat = prm->flattening ? 1 : 0;
     TRYC(cudaMalloc(&P->d_K, sizeof(SchemeConsts)));
-    TRYC(cudaMemcpy(P->d_K, &K, sizeof(SchemeConsts), cudaMemcpyHostToDevice));
+    TRYC(plan_upload(P, P->d_K, &K, sizeof(SchemeConsts)));
     TRYC(cudaMalloc(&P->d_SC, sizeof(StepConsts)));
     TRYC(cudaMalloc(&P->d_BS, sizeof(BoxStep) * P->nbox));
     TRYC(cudaMalloc(&P->d_dtacc, sizeof(unsigned long long)));
     unsigned long long inf = 0x7ff0000000000000ULL;
-    TRYC(cudaMemcpy(P->d_dtacc, &inf, sizeof(inf), cudaMemcpyHostToDevice));
+    TRYC(plan_upload(P, P->d_dtacc, &inf, sizeof(inf)));
     TRYC(cudaMalloc(&P->d_status, sizeof(unsigned)));
-    TRYC(cudaMemset(P->d_status, 0, sizeof(unsigned)));
+    TRYC(plan_upload(P, P->d_status, nullptr, sizeof(unsigned)));
     TRYC(cudaMalloc(&P->d_status_tune, sizeof(unsigned)));
-    TRYC(cudaMemset(P->d_status_tune, 0, sizeof(unsigned)));
+    TRYC(plan_upload(P, P->d_status_tune, nullptr, sizeof(unsigned)));
     TRYC(cudaMalloc(&P->d_scal, 4 * sizeof(double)));
     if (K.flat) {
       const size_t esz = prm->precision == NYX_MIXED ? sizeof(float) : sizeof(double);
@@ -1684,8 +1690,7 @@ int nyx_hydro_plan(const nyx_level_desc *lev, const nyx_hydro_params *prm, void 
       }
       P->flat_ntiles = (int)ft.size();
       TRYC(cudaMalloc(&P->d_flat_tiles, sizeof(FlatTile) * ft.size()));
-      TRYC(cudaMemcpy(P->d_flat_tiles, ft.data(), sizeof(FlatTile) * ft.size(),
-                      cudaMemcpyHostToDevice));
+      TRYC(plan_upload(P, P->d_flat_tiles, ft.data(), sizeof(FlatTile) * ft.size()));
       TRYC((cudaError_t)flatten_init(prm->precision));
       TRYC((cudaError_t)launch_flat_ones(prm->precision, P->d_flat, P->total_stride, P->stream));
       TRYC(cudaStreamSynchronize(P->stream));
@@ -1709,7 +1714,7 @@ int nyx_hydro_plan(const nyx_level_desc *lev, const nyx_hydro_params *prm, void 
       P->shape = prm->precision == NYX_MIXED ? 3 : 0;
       TRY(ensure_items(P, P->shape));
       TRYC(cudaMalloc(&P->d_queue, sizeof(int)));
-      TRYC(cudaMemset(P->d_queue, 0, sizeof(int)));
+      TRYC(plan_upload(P, P->d_queue, nullptr, sizeof(int)));
       TRYC(cudaGetLastError());
     }
     if (prm->keep_fluxes) {
@@ -1723,8 +1728,7 @@ int nyx_hydro_plan(const nyx_level_desc *lev, const nyx_hydro_params *prm, void 
       }
       TRYC(cudaMalloc(&P->d_flux, sizeof(double) * acc));
       TRYC(cudaMalloc(&P->d_flux_off, sizeof(long long) * P->nbox));
-      TRYC(cudaMemcpy(P->d_flux_off, P->flux_off.data(), sizeof(long long) * P->nbox,
-                      cudaMemcpyHostToDevice));
+      TRYC(plan_upload(P, P->d_flux_off, P->flux_off.data(), sizeof(long long) * P->nbox));
     }
   }
   *out = P;
@@ -1909,7 +1913,7 @@ int nyx_hydro_step_host_valid(nyx_plan *P, nyx_level *L, const double *host_in, 
     cudaError_t e = cudaMalloc(&P->d_packed, sizeof(double) * NCONS * (size_t)P->total_cells);
     if (e == cudaSuccess) e = cudaMalloc(&P->d_plane_pref, sizeof(int) * P->nbox);
     if (e == cudaSuccess)
-      e = cudaMemcpy(P->d_plane_pref, pp.data(), sizeof(int) * P->nbox, cudaMemcpyHostToDevice);
+      e = plan_upload(P, P->d_plane_pref, pp.data(), sizeof(int) * P->nbox);
     if (e != cudaSuccess) {
       cudaFree(P->d_packed);
       cudaFree(P->d_plane_pref);
@@ -2070,10 +2074,10 @@ int nyx_hydro_counters_read(nyx_plan *P, int reset, nyx_hydro_counters *out) {
 
 int nyx_hydro_status(nyx_plan *P, int *flags) {
   if (!P) return fail(NYX_EINVAL, "null plan");
-  CK(cudaStreamSynchronize(P->stream));
   unsigned st = 0;
-  CK(cudaMemcpy(&st, P->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost));
-  CK(cudaMemset(P->d_status, 0, sizeof(unsigned)));
+  CK(cudaMemcpyAsync(&st, P->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, P->stream));
+  CK(cudaMemsetAsync(P->d_status, 0, sizeof(unsigned), P->stream));
+  CK(cudaStreamSynchronize(P->stream));
   if (flags) *flags = (int)st;
   if (st & ST_NONFINITE) return fail(NYX_ENONFINITE, "non-finite value in an updated state");
   if (st & ST_NEGATIVE) return fail(NYX_ENEGATIVE, "density <= 0 after an update");

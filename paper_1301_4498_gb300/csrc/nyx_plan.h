@@ -45,6 +45,7 @@ struct nyx_plan {
   std::vector<nyx_domain> doms;
   nyx_hydro_params prm{};
   cudaStream_t stream = nullptr;
+  cudaStream_t up_stream = nullptr;  // tables on their way to the device (plan_upload)
   std::vector<nyx::BoxDev> hbox;
   std::vector<long long> cell_pref;
   long long total_cells = 0;
@@ -160,6 +161,11 @@ struct nyx_plan {
 namespace nyx {
 namespace host {
 
+// Copy a host table to the device (src null: zeros).  It is there when the call
+// returns: a plain cudaMemcpy from pageable memory may return before its last
+// transfer, which nothing orders before kernels on a non-blocking stream, and
+// it joins a capture of a blocking one.
+cudaError_t plan_upload(const nyx_plan *P, void *dst, const void *src, size_t bytes);
 // Ghost fill of a level field, one advance, and the CFL reduction of one
 // plan (all enqueued on the plan's stream; see nyx_api.cu).
 int plan_fill(nyx_plan *P, double *field, int ncomp);

@@ -1346,8 +1346,11 @@ int nyx_poisson_create(nyx_plan *P, const nyx_poisson_params *prm, nyx_poisson *
       rc = fail(NYX_ENOMEM, "Poisson grid allocation failed");
       break;
     }
-    cudaMemset(l.phi, 0, v * sizeof(double));
     S->L.push_back(l);
+    if (plan_upload(P, l.phi, nullptr, v * sizeof(double)) != cudaSuccess) {
+      rc = fail(NYX_ECUDA, "Poisson grid set-up failed");
+      break;
+    }
     if (prm->precision == NYX_MIXED) {
       LevelT<float> l32;
       l32.d = l.d;
@@ -1395,8 +1398,7 @@ int nyx_poisson_create(nyx_plan *P, const nyx_poisson_params *prm, nyx_poisson *
         cudaMalloc(&S->d_scal, sizeof(double) * 2) != cudaSuccess ||
         cudaMalloc(&S->d_max, 2 * sizeof(unsigned long long)) != cudaSuccess)
       rc = fail(NYX_ENOMEM, "Poisson scratch allocation failed");
-    else if (cudaMemcpy(S->d_box_lo, lo.data(), lo.size() * sizeof(int), cudaMemcpyHostToDevice) !=
-             cudaSuccess)
+    else if (plan_upload(P, S->d_box_lo, lo.data(), lo.size() * sizeof(int)) != cudaSuccess)
       rc = fail(NYX_ECUDA, "Poisson table upload failed");
   }
   if (rc) {

@@ -1,6 +1,8 @@
 """What an earlier call leaves in a plan does not change a later one: box
 groups made by a run and by a host step, tile shapes changed between replays
-of a run's graph."""
+of a run's graph, a tile shape chosen while a stream is being captured."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -169,3 +171,32 @@ def test_two_level_graphs_follow_the_tile_shapes():
         assert np.array_equal(W.valid(x), W.valid(y))
     for o in (amr, fp, cp, amq, fq, cq):
         o.close()
+
+
+def test_a_tile_shape_chosen_while_a_stream_is_captured():
+    # a blocking stream: work on the default stream would join the capture
+    w = W.tiled_box(n=64, box=32, nsteps=1)
+    s = C.c_void_p()
+    assert int(torch.cuda.cudart().cudaStreamCreate(C.addressof(s))) == 0
+    stream = torch.cuda.ExternalStream(s.value)
+    plan = _plan(w, stream=stream)
+    lev = H.make_level(plan, w.state, w.grav)
+    a, d = _scalars(1e-5)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        plan.set_tile_shape(5)       # its work list is made and uploaded here
+        plan.advance(lev, a[:1], a[1:2], d[:1])
+    graph.replay()
+    torch.cuda.synchronize()
+    assert plan.status()[0] == H.NYX_OK
+    ref = _plan(w)
+    ref.set_tile_shape(5)
+    rl = H.make_level(ref, w.state, w.grav)
+    ref.advance(rl, a[:1], a[1:2], d[:1])
+    for x, y in zip(plan.from_device(lev.current, 6), ref.from_device(rl.current, 6)):
+        assert np.array_equal(W.valid(x), W.valid(y))
+    del graph
+    plan.close()
+    ref.close()
+    torch.cuda.cudart().cudaStreamDestroy(s.value)
