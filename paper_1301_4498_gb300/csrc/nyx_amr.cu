@@ -69,6 +69,7 @@ struct AvgRect {
 };
 
 constexpr int kMaxGrid = 152 * 16;
+constexpr int kMaxComps = 65535;  // components per launch (the limit of grid y)
 
 // Comparisons on the integer pipe: the FP64 pipe (1/64 of the FP32 rate, and
 // it also compares) bounds the interpolation.  Bit patterns of magnitudes
@@ -106,9 +107,10 @@ __device__ __forceinline__ double mc_slope_d(double sm, double s0, double sp) {
 // (up to 8) fine cells.  The fine values are uc + alpha (+-qx +-qy +-qz) with
 // q = 0.25 slope: rounding is symmetric, so the 8 sums come from 4 with both
 // signs, and each is the value of the cell-by-cell expression.
-__global__ void k_amr_interp(const double *cf, double *ff, int ncomp, const BoxDev *cboxes,
-                             const BoxDev *fboxes, const InterpRect *rects, int nrect) {
-  const int c = blockIdx.y;
+__global__ void k_amr_interp(const double *cf, double *ff, int ncomp, int first,
+                             const BoxDev *cboxes, const BoxDev *fboxes, const InterpRect *rects,
+                             int nrect) {
+  const int c = first + blockIdx.y;
   for (int r = blockIdx.x; r < nrect; r += gridDim.x) {
     const InterpRect R = rects[r];
     const BoxDev &bc = cboxes[R.cbox];
@@ -234,9 +236,10 @@ __global__ void k_amr_reflux(double *cs, const double *cflux, const long long *c
   }
 }
 
-__global__ void k_amr_avgdown(const double *ff, double *cf, int ncomp, const BoxDev *cboxes,
-                              const BoxDev *fboxes, const AvgRect *rects, int nrect) {
-  const int c = blockIdx.y;
+__global__ void k_amr_avgdown(const double *ff, double *cf, int ncomp, int first,
+                              const BoxDev *cboxes, const BoxDev *fboxes, const AvgRect *rects,
+                              int nrect) {
+  const int c = first + blockIdx.y;
   for (int r = blockIdx.x; r < nrect; r += gridDim.x) {
     const AvgRect R = rects[r];
     const BoxDev bc = cboxes[R.cbox];
@@ -641,18 +644,22 @@ int enqueue_interp(nyx_amr *A, const double *cf, double *ff, int ncomp, int regi
   const InterpRect *r = region == NYX_AMR_ALL ? A->d_ia : A->d_ig;
   const int n = region == NYX_AMR_ALL ? A->n_ia : A->n_ig;
   if (!n) return NYX_OK;
-  k_amr_interp<<<dim3(grid_of(n), ncomp), 256, 0, C.stream>>>(cf, ff, ncomp, C.d_boxes, F.d_boxes,
-                                                              r, n);
-  C.launches += 1;
+  for (int c = 0; c < ncomp; c += kMaxComps) {
+    k_amr_interp<<<dim3(grid_of(n), std::min(ncomp - c, kMaxComps)), 256, 0, C.stream>>>(
+        cf, ff, ncomp, c, C.d_boxes, F.d_boxes, r, n);
+    C.launches += 1;
+  }
   return NYX_OK;
 }
 
 int enqueue_avgdown(nyx_amr *A, const double *ff, double *cf, int ncomp) {
   nyx_plan &C = *A->C, &F = *A->F;
   if (!A->n_avg) return NYX_OK;
-  k_amr_avgdown<<<dim3(grid_of(A->n_avg), ncomp), 256, 0, C.stream>>>(
-      ff, cf, ncomp, C.d_boxes, F.d_boxes, A->d_avg, A->n_avg);
-  C.launches += 1;
+  for (int c = 0; c < ncomp; c += kMaxComps) {
+    k_amr_avgdown<<<dim3(grid_of(A->n_avg), std::min(ncomp - c, kMaxComps)), 256, 0, C.stream>>>(
+        ff, cf, ncomp, c, C.d_boxes, F.d_boxes, A->d_avg, A->n_avg);
+    C.launches += 1;
+  }
   return NYX_OK;
 }
 

@@ -269,3 +269,24 @@ def test_mixed_poisson_on_a_long_domain(warm):
             <= 0.26 * (per * h)**2 * 1e-12 * np.abs(f).max() + 1e-12 * np.abs(ref).max())
     ps.close()
     plan.close()
+
+
+def test_interpolation_and_average_down_of_more_components_than_a_grid_holds():
+    # components run along grid y, of at most 65535 blocks: two fields in turn
+    n = 70000
+    cl = W.single_box_level(8, 8, 8, 1.0 / 8)
+    fl = W.refined_level(cl, [(0, (2, 2, 2), (3, 3, 3))])
+    cp = H.Plan(cl, precision="fp64", keep_fluxes=1)
+    fp = H.Plan(fl, stream=cp.torch_stream, precision="fp64", keep_fluxes=1, coarse_fine=1)
+    amr = H.Amr(cp, fp)
+    c2 = cp.empty_field(2)
+    c2.copy_(torch.rand(c2.shape, dtype=torch.float64, device="cuda"))
+    f2, back = fp.empty_field(2), cp.empty_field(2)
+    amr.interp(c2, f2, 2, "all")
+    amr.average_down(f2, back, 2)
+    cn = c2.repeat(n // 2)            # one box: components follow one another
+    fn, bn = fp.empty_field(n), cp.empty_field(n)
+    amr.interp(cn, fn, n, "all")
+    amr.average_down(fn, bn, n)
+    assert torch.equal(fn, f2.repeat(n // 2)) and torch.equal(bn, back.repeat(n // 2))
+    amr.close(); fp.close(); cp.close()
