@@ -965,6 +965,9 @@ struct nyx_poisson {
   // fixed-point potential of the refinement solve (while `fixed`): units of
   // 1/fix_s, at most (fix_top + 1) 2^32 of them; h^2 times the right-hand side
   // is then fixed point in L[0].f's memory, in units of 1/(fix_s 2^fix_k)
+  // mixed precision: fused sweeps and fixed point (at least one sweep on each
+  // side, and memory for the second arrays and d_fix)
+  bool fused = false;
   long long *d_fix = nullptr;
   bool fixed = false;
   float fix_s = 0.0f;
@@ -1195,8 +1198,6 @@ void vcycle_fused(nyx_poisson *S) {
   }
 }
 
-bool fused_cycle(const nyx_poisson *S) { return S->prm.pre >= 1 && S->prm.post >= 1; }
-
 // Max norm of the finest grid's residual, and with pmax (mixed precision, phi
 // in FP64) the largest |phi|.
 int resid_max(nyx_poisson *S, double *out, double *pmax = nullptr) {
@@ -1277,7 +1278,7 @@ void cycle(nyx_poisson *S) {
     vcycle(S, S->L, 0, S->tail64, S->targs64);
     return;
   }
-  if (fused_cycle(S)) {
+  if (S->fused) {
     vcycle_fused(S);
     return;
   }
@@ -1287,6 +1288,27 @@ void cycle(nyx_poisson *S) {
   const long long n = (long long)g.d.n[0] * g.d.n[1] * g.d.n[2];
   k_pg_correct<<<gridn(n, 256), 256, 0, S->P->stream>>>(g.phi, S->L32[0].phi, n);
   S->launches += 1;
+}
+
+// Memory of the fused sweeps and the fixed-point potential, 12.6 B a cell beside
+// the grids' 27; without it the solve runs unfused with FP64 residuals.
+bool alloc_fused(nyx_poisson *S) {
+  const auto cells = [](const LevelT<float> &g) {
+    return (size_t)g.d.n[0] * g.d.n[1] * g.d.n[2];
+  };
+  bool ok = cudaMalloc(&S->d_fix, cells(S->L32[0]) * sizeof(long long)) == cudaSuccess;
+  const size_t nl = std::min(S->tail32, S->L32.size());
+  for (size_t l = 0; ok && l < nl; ++l)
+    ok = cudaMalloc(&S->L32[l].phi2, cells(S->L32[l]) * sizeof(float)) == cudaSuccess;
+  if (ok) return true;
+  cudaGetLastError();
+  cudaFree(S->d_fix);
+  S->d_fix = nullptr;
+  for (auto &g : S->L32) {
+    cudaFree(g.phi2);
+    g.phi2 = nullptr;
+  }
+  return false;
 }
 
 }  // namespace
@@ -1376,16 +1398,7 @@ int nyx_poisson_create(nyx_plan *P, const nyx_poisson_params *prm, nyx_poisson *
     if (!S->L32.empty()) {
       S->tail32 = make_tail(S, S->L32, 0, S->targs32, S->tsmem32);
       rc = smooth_init();
-      if (!rc && fused_cycle(S) &&
-          cudaMalloc(&S->d_fix, sizeof(long long) * (size_t)n[0] * n[1] * n[2]) != cudaSuccess)
-        rc = fail(NYX_ENOMEM, "Poisson grid allocation failed");
-      if (fused_cycle(S))
-        for (size_t l = 0; l < std::min(S->tail32, S->L32.size()) && !rc; ++l) {
-          LevelT<float> &g = S->L32[l];
-          const size_t v = (size_t)g.d.n[0] * g.d.n[1] * g.d.n[2];
-          if (cudaMalloc(&g.phi2, v * sizeof(float)) != cudaSuccess)
-            rc = fail(NYX_ENOMEM, "Poisson grid allocation failed");
-        }
+      if (!rc && prm->pre >= 1 && prm->post >= 1) S->fused = alloc_fused(S);
     }
   }
   if (!rc) {
