@@ -77,29 +77,28 @@ __global__ void k_estdt_mixed(const BoxDev *boxes, const long long *cell_pref, i
   const float small_pres = nyx_mixed::d2f_rn(K->small_pres);
   const double a = *a_dev;
   float local_min = __int_as_float(0x7f800000);
-  int box = -1;
-  float adx[3] = {0.0f, 0.0f, 0.0f};  // a dx of the current box (FP64 products)
-  for (CellWalk w(cell_pref, nbox, total); w.valid(); w.next(cell_pref, nbox)) {
-    const BoxDev &b = boxes[w.box];
-    if (w.box != box) {
-      box = w.box;
+  for (CellWalk w(cell_pref, nbox, total); w.valid(); w.find(cell_pref, nbox)) {
+    const BoxDev b = boxes[w.box];
+    const long long e = w.box_end(cell_pref, nbox);
+    float adx[3];
 #pragma unroll
-      for (int d = 0; d < 3; ++d) adx[d] = (float)(a * b.dx[d]);
-    }
-    int i, j, kk;
-    w.cell(cell_pref, b, i, j, kk);
-    const double *S = state + NCONS * b.pref;
-    const long long id = cell_index(b, i, j, kk);
-    const float rho = nyx_mixed::d2f_rn(S[id]);
-    const float ir = 1.0f / rho;
-    float p = gm1 * nyx_mixed::d2f_rn(S[5 * b.stride + id]);
-    if (p < small_pres) p = small_pres;
-    const float c2 = gamma * p * ir;
-    const float c = c2 * rsqrtf(c2);
+    for (int d = 0; d < 3; ++d) adx[d] = nyx_mixed::d2f_rn(a * b.dx[d]);
+    for (; w.t < e; w.t += blockDim.x) {
+      int i, j, kk;
+      w.cell(cell_pref, b, i, j, kk);
+      const double *S = state + NCONS * b.pref;
+      const long long id = cell_index(b, i, j, kk);
+      const float rho = nyx_mixed::d2f_rn(S[id]);
+      const float ir = 1.0f / rho;
+      float p = gm1 * nyx_mixed::d2f_rn(S[5 * b.stride + id]);
+      if (p < small_pres) p = small_pres;
+      const float c2 = gamma * p * ir;
+      const float c = c2 * rsqrtf(c2);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const float tt = adx[d] / (fabsf(nyx_mixed::d2f_rn(S[(1 + d) * b.stride + id]) * ir) + c);
-      local_min = fminf(local_min, tt);
+      for (int d = 0; d < 3; ++d) {
+        const float tt = adx[d] / (fabsf(nyx_mixed::d2f_rn(S[(1 + d) * b.stride + id]) * ir) + c);
+        local_min = fminf(local_min, tt);
+      }
     }
   }
   for (int o = 16; o > 0; o >>= 1) local_min = fminf(local_min, __shfl_xor_sync(0xffffffffu, local_min, o));

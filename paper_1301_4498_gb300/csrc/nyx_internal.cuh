@@ -105,7 +105,20 @@ struct CellWalk {
   __device__ __forceinline__ bool valid() const { return t < end; }
   __device__ __forceinline__ void next(const long long *cell_pref, int nbox) {
     t += blockDim.x;
+    find(cell_pref, nbox);
+  }
+  // ... or box by box: for (; valid(); find()) for (; t < box_end(); t += blockDim.x),
+  // with what depends on the box alone formed once, ahead of the inner loop (in
+  // the one loop a test for a new box does not keep it out of every cell's work:
+  // the FP64 products a dx made the mixed CFL pass 291 us for 256^3 cells, 194 us
+  // before the walk)
+  __device__ __forceinline__ void find(const long long *cell_pref, int nbox) {
     while (box + 1 < nbox && cell_pref[box + 1] <= t) ++box;
+  }
+  __device__ __forceinline__ long long box_end(const long long *cell_pref, int nbox) const {
+    if (box + 1 >= nbox) return end;
+    const long long e = cell_pref[box + 1];
+    return e < end ? e : end;
   }
   // local cell of the current box
   __device__ __forceinline__ void cell(const long long *cell_pref, const BoxDev &b, int &i, int &j,

@@ -420,20 +420,24 @@ __global__ void k_estdt(const BoxDev *boxes, const long long *cell_pref, int nbo
   const SchemeConsts k = *K;
   const double a = *a_dev;
   double local_min = __longlong_as_double(0x7ff0000000000000LL);
-  for (CellWalk w(cell_pref, nbox, total); w.valid(); w.next(cell_pref, nbox)) {
-    const BoxDev &b = boxes[w.box];
-    int i, j, kk;
-    w.cell(cell_pref, b, i, j, kk);
-    const double *S = state + NCONS * b.pref;
-    long long id = cell_index(b, i, j, kk);
-    const double rho = S[id];
-    double p = k.gm1 * S[5 * b.stride + id];
-    if (p < k.small_pres) p = k.small_pres;
-    const double c = sqrt(k.gamma * p / rho);
+  for (CellWalk w(cell_pref, nbox, total); w.valid(); w.find(cell_pref, nbox)) {
+    const BoxDev b = boxes[w.box];
+    const long long e = w.box_end(cell_pref, nbox);
+    const double adx[3] = {a * b.dx[0], a * b.dx[1], a * b.dx[2]};
+    for (; w.t < e; w.t += blockDim.x) {
+      int i, j, kk;
+      w.cell(cell_pref, b, i, j, kk);
+      const double *S = state + NCONS * b.pref;
+      long long id = cell_index(b, i, j, kk);
+      const double rho = S[id];
+      double p = k.gm1 * S[5 * b.stride + id];
+      if (p < k.small_pres) p = k.small_pres;
+      const double c = sqrt(k.gamma * p / rho);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      double tt = a * b.dx[d] / (fabs(S[(1 + d) * b.stride + id] / rho) + c);
-      if (tt < local_min) local_min = tt;
+      for (int d = 0; d < 3; ++d) {
+        double tt = adx[d] / (fabs(S[(1 + d) * b.stride + id] / rho) + c);
+        if (tt < local_min) local_min = tt;
+      }
     }
   }
   for (int o = 16; o > 0; o >>= 1) {
