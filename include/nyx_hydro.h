@@ -207,9 +207,9 @@ int nyx_hydro_correct(nyx_plan *plan, nyx_level *level, const double *a_old_dev,
  * nyx_hydro_estdt if compute_dt0 != 0) and step s writes dt_dev[s+1].
  * use_graph != 0 captures the sequence once into a CUDA graph (kept in the
  * plan, keyed by the pointers and nsteps) and replays it.  On a persistent
- * plan whose level has enough work items (4 waves or more) the boxes are cut
- * into the groups of nyx_hydro_step_host_valid (made on the first call):
- * every step runs one advance launch per group, and each group's ghost fill
+ * plan whose level has enough work items (8 waves of the task form's, 4 of
+ * the column-owning form's) the boxes are cut into groups (made on the first
+ * call once the plan is tuned): every step runs one advance launch per group, and each group's ghost fill
  * of the next step starts as soon as the groups it reads have advanced,
  * beside the other groups' advances (a flattening plan's coefficient pass
  * then runs over the whole level before the step's advances).  The result is
@@ -260,7 +260,8 @@ int nyx_hydro_step_host_valid(nyx_plan *plan, nyx_level *level, const double *ho
  * mixed), 3-5 the task form (mixed only).  nyx_hydro_tile_shape returns
  * NYX_EINVAL for an index out of range; nyx_hydro_set_tile_shape fixes the
  * plan's shape (and turns its autotuner off; NYX_EINVAL if the shape does
- * not exist for the plan's precision); nyx_hydro_get_tile_shape reports the
+ * not exist for the plan's precision; graphs the plan keeps are recorded
+ * again); nyx_hydro_get_tile_shape reports the
  * shape in use. */
 int nyx_hydro_tile_shape(int shape, int *tx, int *ty);
 int nyx_hydro_set_tile_shape(nyx_plan *plan, int shape);
@@ -286,7 +287,9 @@ int nyx_hydro_tune_info(const nyx_plan *plan, int *classes, int *trials, int *la
 /* Work list of the fused persistent kernel for a level of nbox boxes with
  * interior extents n[3b], n[3b+1], n[3b+2] (x, y, z) and column tiles of
  * tx x ty, run on `slots` resident CTAs that take items from one queue.
- * Host only: it needs no GPU and no plan, and is the list a plan builds.
+ * Host only: it needs no GPU and no plan, and is the list a plan builds for
+ * a tile of the task form (the column-owning form runs its whole tile width
+ * at the box edge too, and its lists weigh items so).
  * Each item is 7 ints (box, x0, y0, nx, ny, z0, nz): cells [x0, x0+nx) x
  * [y0, y0+ny) x [z0, z0+nz) of the box; the items tile every box once.
  * chunk = 0 keeps every column whole; chunk != 0 lets the list cut columns
@@ -384,16 +387,19 @@ typedef struct {
   int min_size;       /* smallest coarse extent (2) */
   double four_pi_G;   /* 4 pi G in code units (1) */
   int precision;      /* NYX_FP64 (default): every operation in FP64.  NYX_MIXED:
-                         iterative refinement, each cycle an FP64 residual, one
-                         FP32 V-cycle on the correction equation from zero, and
-                         an FP64 update of phi; the stopping test on that
-                         FP64 residual, rounded to float */
+                         iterative refinement, each cycle a residual, one FP32
+                         V-cycle on the correction equation from zero, and the
+                         update of phi, residual sums and phi in 64-bit fixed
+                         point (FP64 where no scale fits, without a pre- or a
+                         post-sweep, or without memory for it); the stopping
+                         test on that residual, rounded to float */
 } nyx_poisson_params;
 
 void nyx_poisson_default_params(nyx_poisson_params *params);
 
-/* Check the plan's level and allocate the grids (about 2.3 doubles per
- * cell).  NYX_EINVAL if the level cannot be solved this way. */
+/* Check the plan's level and allocate the grids (about 2.3 doubles per cell;
+ * NYX_MIXED 3.4, and 1.6 more for fused sweeps and fixed point where they
+ * fit).  NYX_EINVAL if the level cannot be solved this way. */
 int nyx_poisson_create(nyx_plan *plan, const nyx_poisson_params *params, nyx_poisson **out);
 
 /* Solve for the state (device field, 6 components, rho first) plus rho_dm

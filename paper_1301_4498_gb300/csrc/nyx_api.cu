@@ -1340,9 +1340,10 @@ int run_grouped(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev, 
       CK(cudaEventRecord(B.ev_ready[g], fs));
     }
     if (P->d_flat) {
-      // the coefficient pass (512 threads, 43 KB of shared memory per block)
-      // does not fit beside the advance: it runs over the whole level once
-      // every group is filled, before the step's advances
+      // the coefficient pass (in FP32 320 threads of 40 registers and 43 KB of
+      // shared memory per block) does not fit beside the advance (203 KB and
+      // 60 K of the 64 K registers): it runs over the whole level once every
+      // group is filled, before the step's advances
       for (int k = 0; k < 2; ++k) {
         CK(cudaEventRecord(P->ev_fjoin[k], P->fill_stream[k]));
         CK(cudaStreamWaitEvent(P->stream, P->ev_fjoin[k], 0));
@@ -1806,7 +1807,7 @@ int nyx_hydro_run(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev
     // possible without the caller's buffers, so tune on the real ones and
     // redo the work below (the tuning launches only write state[1-cur]).
     FusedArgs a{};
-      a.boxes = P->d_boxes;
+    a.boxes = P->d_boxes;
     a.queue = P->d_queue;
     a.K = P->d_K;
     a.SC = P->d_SC;

@@ -471,40 +471,30 @@ __global__ void k_pg_shift_fix(long long *y, long long n, int b) {
 // rounding to float; c = 1 / (h^2 s).
 //
 // Bound: memory.  A thread marches zc planes with the cells above and below in
-// registers, two cells of a row at a time where rows are even (PAIR): 19 B a
-// cell from L2.  One thread per cell read 59 B a cell: 164 us on a 256^3 grid
+// registers, two cells of a row at a time (rows are even): 19 B a cell from L2.  One thread per cell read 59 B a cell: 164 us on a 256^3 grid
 // (324 MB of DRAM), 86 us this way.
 constexpr int kRfX = 32, kRfY = 8;
-template <bool PAIR>
 __global__ void __launch_bounds__(kRfX *kRfY)
     k_pg_resid_fix(const unsigned long long *phi, const long long *f, Dims d, float c, int K,
                    int zc, float *r, unsigned long long *out) {
-  constexpr int W = PAIR ? 2 : 1;
   struct Cells {
-    unsigned long long v[W];
+    unsigned long long v[2];
   };
   auto load = [](const void *p, long long t) {
-    Cells q;
-    if (PAIR) {
-      const ulonglong2 w = reinterpret_cast<const ulonglong2 *>(p)[t >> 1];
-      q.v[0] = w.x;
-      q.v[W - 1] = w.y;
-    } else {
-      q.v[0] = reinterpret_cast<const unsigned long long *>(p)[t];
-    }
-    return q;
+    const ulonglong2 w = reinterpret_cast<const ulonglong2 *>(p)[t >> 1];
+    return Cells{{w.x, w.y}};
   };
   float loc = 0.0f;
   unsigned pm = 0;
   const int nx = d.n[0], ny = d.n[1], nz = d.n[2];
-  const int i = (blockIdx.x * kRfX + threadIdx.x) * W, j = blockIdx.y * kRfY + threadIdx.y;
+  const int i = (blockIdx.x * kRfX + threadIdx.x) * 2, j = blockIdx.y * kRfY + threadIdx.y;
   const int z0 = blockIdx.z * zc, z1 = min(nz, z0 + zc);
   if (i < nx && j < ny) {
     const long long sz = (long long)nx * ny;
     const long long o = (long long)j * nx + i;
     const long long ym = (long long)(j ? j - 1 : ny - 1) * nx + i;
     const long long yp = (long long)(j + 1 < ny ? j + 1 : 0) * nx + i;
-    const long long xm = i ? o - 1 : o + nx - 1, xp = i + W < nx ? o + W : o + W - nx;
+    const long long xm = i ? o - 1 : o + nx - 1, xp = i + 2 < nx ? o + 2 : o + 2 - nx;
     const float cK = c * __int_as_float((127 - K) << 23);
     const unsigned long long lim = 1ull << (62 - K);
     Cells lo = load(phi, (z0 ? z0 - 1 : nz - 1) * sz + o), mid = load(phi, z0 * sz + o);
@@ -513,10 +503,10 @@ __global__ void __launch_bounds__(kRfX *kRfY)
       const Cells hi = load(phi, (k + 1 < nz ? zb + sz : 0) + o);
       const Cells a = load(phi, zb + ym), b = load(phi, zb + yp), ff = load(f, zb + o);
       const unsigned long long left = phi[zb + xm], right = phi[zb + xp];
-      float q[W];
+      float q[2];
 #pragma unroll
-      for (int u = 0; u < W; ++u) {
-        const unsigned long long w = u == 0 ? left : mid.v[0], e = u == W - 1 ? right : mid.v[W - 1];
+      for (int u = 0; u < 2; ++u) {
+        const unsigned long long w = u == 0 ? left : mid.v[0], e = u == 0 ? mid.v[1] : right;
         const unsigned long long nb = w + e + a.v[u] + b.v[u] + lo.v[u] + hi.v[u];
         const long long F = (long long)ff.v[u];
         const unsigned long long v = (unsigned long long)(F >> K) + 6 * mid.v[u] - nb;
@@ -527,10 +517,7 @@ __global__ void __launch_bounds__(kRfX *kRfY)
         const int top = (int)(mid.v[u] >> 32);
         pm = max(pm, (unsigned)(top ^ (top >> 31)));
       }
-      if (PAIR)
-        *reinterpret_cast<float2 *>(r + zb + o) = make_float2(q[0], q[W - 1]);
-      else
-        r[zb + o] = q[0];
+      *reinterpret_cast<float2 *>(r + zb + o) = make_float2(q[0], q[1]);
       lo = mid;
       mid = hi;
     }
@@ -1095,7 +1082,6 @@ void vcycle(nyx_poisson *S, std::vector<LevelT<T>> &L, size_t l, size_t tail_at,
   for (int s = 0; s < S->prm.post; ++s) sweep(S, g);
 }
 
-// One fused sweep of FP32 grid l from phi_in into phi_out.
 // Planes per CTA of the fused sweeps: even (a coarse plane stays in one CTA).  A
 // CTA takes 7 steps more than planes, and a step about 1 us alone on an SM, 1.42
 // and 1.85 us with one or two others (three fit; 128^3 grid); of the even
@@ -1116,6 +1102,7 @@ int smooth_planes(int tiles, int nz) {
   return best;
 }
 
+// One fused sweep of FP32 grid l from `in` into `out`.
 template <bool ZERO, bool PROLONG, bool RESTRICT, int ADD>
 void smooth_launch(nyx_poisson *S, size_t l, const float *in, float *out, const float *pc) {
   const LevelT<float> &g = S->L32[l];
@@ -1206,12 +1193,11 @@ int resid_max(nyx_poisson *S, double *out, double *pmax = nullptr) {
   CK(cudaMemsetAsync(S->d_max, 0, 2 * sizeof(unsigned long long), S->P->stream));
   if (S->fixed) {
     LevelT<float> &g32 = S->L32[0];
-    const int w = g.d.n[0] % 2 ? 1 : 2;
-    dim3 G((g.d.n[0] + kRfX * w - 1) / (kRfX * w), (g.d.n[1] + kRfY - 1) / kRfY);
+    dim3 G((g.d.n[0] / 2 + kRfX - 1) / kRfX, (g.d.n[1] + kRfY - 1) / kRfY);
     // planes per CTA: 16 (one in 8 read again), fewer while that leaves SMs idle
     const int zc = (int)std::min(16ll, std::max(2ll, (long long)G.x * G.y * g.d.n[2] / (152 * 8)));
     G.z = (g.d.n[2] + zc - 1) / zc;
-    (w == 2 ? k_pg_resid_fix<true> : k_pg_resid_fix<false>)<<<G, dim3(kRfX, kRfY), 0, S->P->stream>>>(
+    k_pg_resid_fix<<<G, dim3(kRfX, kRfY), 0, S->P->stream>>>(
         (const unsigned long long *)S->d_fix, (const long long *)g.f, g.d,
         (float)(g.ih2 / (double)S->fix_s), S->fix_k, zc, g32.f, S->d_max);
   } else if (S->L32.empty()) {
@@ -1271,8 +1257,8 @@ void refine_fixed(nyx_poisson *S, double res) {
 }
 
 // One cycle: a V-cycle on phi (FP64), or a refinement step (FP32 V-cycle on
-// the correction equation whose right-hand side resid_max left, then phi +=
-// e in FP64).
+// the correction equation whose right-hand side resid_max left, then phi += e,
+// in fixed point or FP64).
 void cycle(nyx_poisson *S) {
   if (S->L32.empty()) {
     vcycle(S, S->L, 0, S->tail64, S->targs64);
