@@ -184,14 +184,18 @@ __device__ __forceinline__ long long flux_block(const BoxDev &b, int d, int e[3]
   return off;
 }
 
+// One thread per coarse face cell: of one component (SPLIT, grid y) where the
+// faces are few, else of all six, so that its indices and the mask are formed
+// once.  Six launches, by the number of refined 32^3 boxes (one component /
+// all six, us): 6 41 / 54, 24 92 / 86, 51 182 / 150, 410 1254 / 920.
+template <bool SPLIT>
 __global__ void k_amr_reflux(double *cs, const double *cflux, const long long *cflux_off,
                              const double *fflux, const long long *fflux_off,
                              const BoxDev *cboxes, const BoxDev *fboxes,
                              const unsigned char *covered, const long long *ccell_pref,
                              const StepConsts *SC, const FaceRect *rects, int nrect) {
   const StepConsts sc = *SC;
-  const int c = blockIdx.y;
-  const double coef = c == 0 ? sc.dtp : (c < 4 ? sc.dt * sc.ian : sc.ahdt * sc.ian2);
+  const double coef[3] = {sc.dtp, sc.dt * sc.ian, sc.ahdt * sc.ian2};  // rho, m, energies
   for (int r = blockIdx.x; r < nrect; r += gridDim.x) {
     const FaceRect R = rects[r];
     const BoxDev bc = cboxes[R.cbox];
@@ -218,20 +222,24 @@ __global__ void k_amr_reflux(double *cs, const double *cflux, const long long *c
       const long long cid = ((long long)cfi[2] * ce[1] + cfi[1]) * ce[0] + cfi[0];
       const long long sid = cell_index(bc, P[0], P[1], P[2]);
       const int f1 = R.ft0[0] + 2 * a1, f2 = R.ft0[1] + 2 * a2;
-      double fsum = 0.0;
 #pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        int fi[3];
-        fi[d] = ffi;
-        fi[t1] = f1 + (s & 1);
-        fi[t2] = f2 + (s >> 1);
-        const double v = Ff[c * fv + ((long long)fi[2] * fe[1] + fi[1]) * fe[0] + fi[0]];
-        fsum = (s == 0) ? v : fsum + v;
+      for (int u = 0; u < (SPLIT ? 1 : 6); ++u) {
+        const int c = SPLIT ? (int)blockIdx.y : u;
+        double fsum = 0.0;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          int fi[3];
+          fi[d] = ffi;
+          fi[t1] = f1 + (s & 1);
+          fi[t2] = f2 + (s >> 1);
+          const double v = Ff[c * fv + ((long long)fi[2] * fe[1] + fi[1]) * fe[0] + fi[0]];
+          fsum = (s == 0) ? v : fsum + v;
+        }
+        const double favg = 0.25 * fsum;
+        const double corr = coef[c == 0 ? 0 : (c < 4 ? 1 : 2)] * ((favg - Fc[c * cv + cid]) * idx);
+        double *u_ = U + c * bc.stride + sid;
+        *u_ = R.high ? *u_ + corr : *u_ - corr;
       }
-      const double favg = 0.25 * fsum;
-      const double corr = coef * ((favg - Fc[c * cv + cid]) * idx);
-      double *u_ = U + c * bc.stride + sid;
-      *u_ = R.high ? *u_ + corr : *u_ - corr;
     }
   }
 }
@@ -433,14 +441,15 @@ struct Builder {
 };
 
 // Rectangles are cut so that small hierarchies still give every SM work: one
-// CTA takes a rectangle and one component, in one or two passes of its
-// threads.  Interpolation rectangles are cut along z at coarse cell boundaries
+// CTA takes a rectangle and one component (reflux of many faces: all of them),
+// in one or two passes of its threads.  Interpolation rectangles are cut along z at coarse cell boundaries
 // (each coarse cell stays in one piece), face and average rectangles along
 // their slowest axis.  Six refined boxes of 64^3, with rectangles of 4096 cells
 // and all components in one CTA and after: ghost cells 397 -> 103 us, average
 // down 210 -> 26 us, reflux 6 x 67 -> 6 x 7.7 us.
 constexpr int kFineChunk = 2048;   // fine cells: 256 coarse ones, a thread each
 constexpr int kFaceChunk = 128;    // coarse face cells
+constexpr int kFewFaces = 192;     // face rectangles below which reflux splits the components
 constexpr int kAvgChunk = 512;     // coarse cells
 
 void split_interp(const InterpRect &R, std::vector<InterpRect> &out) {
@@ -631,7 +640,9 @@ int enqueue_reflux(nyx_amr *A, double *coarse_new) {
   nyx_plan &C = *A->C, &F = *A->F;
   for (int o = 0; o < 6; ++o) {
     if (!A->n_face[o]) continue;
-    k_amr_reflux<<<dim3(grid_of(A->n_face[o]), 6), 128, 0, C.stream>>>(
+    const bool few = A->n_face[o] < kFewFaces;
+    (few ? k_amr_reflux<true> : k_amr_reflux<false>)<<<dim3(grid_of(A->n_face[o]), few ? 6 : 1),
+                                                       128, 0, C.stream>>>(
         coarse_new, C.d_flux, C.d_flux_off, F.d_flux, F.d_flux_off, C.d_boxes, F.d_boxes, A->d_cov,
         C.d_cell_pref, C.d_SC, A->d_face[o], A->n_face[o]);
     C.launches += 1;
