@@ -1110,8 +1110,8 @@ def run_cosmo(args, w):
     if args.tile_shape >= 0:
         plan.set_tile_shape(args.tile_shape)
     lev = H.make_level(plan, w.state, None)
-    # mixed plans solve by iterative refinement (FP64 residual and update
-    # around FP32 V-cycles), to the same FP64 stopping test
+    # mixed plans solve by iterative refinement (residual and update in fixed point
+    # or FP64 around FP32 V-cycles), to the same stopping test
     ps = H.Poisson(plan, four_pi_G=COSMO_FOUR_PI_G, precision=args.precision)
     xd, ud, md = (torch.tensor(v, device="cuda") for v in (x, u, m))
     rho = ps.dense(1)[0]
@@ -1204,7 +1204,7 @@ def run_cosmo(args, w):
             "config": {"workload": args.workload, "level": w.name, "valid_cells": cells,
                        "particles": npart, "boxes": w.level.nbox, "precision": args.precision,
                        "step": "Sec. 3.6 Steps 1-6 (g^n from the previous Step 4)",
-                       "poisson": ("iterative refinement: FP64 residual and update, FP32 "
+                       "poisson": ("iterative refinement: fixed-point residual and update, FP32 "
                                    "V-cycles" if args.precision == "mixed"
                                    else "FP64 V-cycles"),
                        "tile": [tx, ty], "l2": "inputs larger than L2",

@@ -442,9 +442,9 @@ struct Builder {
 
 // Rectangles are cut so that small hierarchies still give every SM work: one
 // CTA takes a rectangle and one component (reflux of many faces: all of them),
-// in one or two passes of its threads.  Interpolation rectangles are cut along z at coarse cell boundaries
-// (each coarse cell stays in one piece), face and average rectangles along
-// their slowest axis.  Six refined boxes of 64^3, with rectangles of 4096 cells
+// in one or two passes of its threads.  Interpolation rectangles are cut along
+// z at coarse cell boundaries (each coarse cell stays in one piece), face and
+// average rectangles along their slowest axis.  Six refined boxes of 64^3, with rectangles of 4096 cells
 // and all components in one CTA and after: ghost cells 397 -> 103 us, average
 // down 210 -> 26 us, reflux 6 x 67 -> 6 x 7.7 us.
 constexpr int kFineChunk = 2048;   // fine cells: 256 coarse ones, a thread each

@@ -1340,7 +1340,7 @@ int run_grouped(nyx_plan *P, nyx_level *L, const double *a_dev, double *dt_dev, 
       CK(cudaEventRecord(B.ev_ready[g], fs));
     }
     if (P->d_flat) {
-      // the coefficient pass (in FP32 320 threads of 40 registers and 43 KB of
+      // the coefficient pass (in FP32 320 threads of 32 registers and 43 KB of
       // shared memory per block) does not fit beside the advance (203 KB and
       // 60 K of the 64 K registers): it runs over the whole level once every
       // group is filled, before the step's advances

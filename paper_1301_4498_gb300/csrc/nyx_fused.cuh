@@ -712,7 +712,7 @@ constexpr int FLAT_TX = 34, FLAT_TY = 17;  // largest output tile
 constexpr int FLAT_NO = FLAT_TX * FLAT_TY;
 constexpr int FLAT_NF = (FLAT_TX + 6) * (FLAT_TY + 6);
 // Five blocks fit an SM in FP32 (43.4 KB of shared memory each) at 320 threads
-// of 40 registers: the planes of one block load while others compute (one
+// of 32 registers: the planes of one block load while others compute (one
 // 192^3 box: 257 us; 385 us with 512 threads, which fitted twice).
 constexpr int FLAT_THREADS = 320;
 

@@ -475,7 +475,7 @@ __global__ void k_pg_shift_fix(long long *y, long long n, int b) {
 //
 // Bound: memory.  A thread marches zc planes with the cells above and below in
 // registers, two cells of a row at a time (rows are even): 19 B a cell from L2.  One thread per cell read 59 B a cell: 164 us on a 256^3 grid
-// (324 MB of DRAM), 86 us this way.
+// (324 MB of DRAM), 90 us this way.
 constexpr int kRfX = 32, kRfY = 8;
 __global__ void __launch_bounds__(kRfX *kRfY)
     k_pg_resid_fix(const unsigned long long *phi, const long long *f, Dims d, float c, int K,

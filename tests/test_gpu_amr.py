@@ -225,3 +225,26 @@ def test_two_level_step_with_flattening_fp64():
     assert _norm_rel(cp.from_device(lc.current, 6), cn) <= 1e-12
     assert _norm_rel(fp.from_device(lf.current, 6), fn) <= 1e-12
     amr.close(); fp.close(); cp.close()
+
+
+def test_reflux_of_many_faces_fp64_matches_the_oracle():
+    # every other 8^3 box of 64^3 refined: 256 faces an orientation, enough for
+    # reflux to take all components in one CTA
+    w = W.tiled_box(n=64, box=8, sigma=0.6, seed=4, nsteps=1)
+    fine = W.refine_boxes(w.level, [b for b in range(w.level.nbox)
+                                    if sum(int(v) // 8 for v in w.level.lo[b]) % 2 == 0])
+    cp, fp, amr, lc, lf = _setup(w, fine, grav=False)
+    cs, fs, cg, fg = _oracle_setup(w, fine, grav=False)
+    P = oracle.OracleParams(gamma=w.gamma, cfl=w.cfl)
+    a0, a1 = float(w.a_sched[0]), float(w.a_sched[1])
+    a = torch.tensor([a0, a1], dtype=torch.float64, device="cuda")
+    dt = torch.zeros(2, dtype=torch.float64, device="cuda")
+    amr.estdt(lc, lf, a[:1], dt[:1])
+    amr.step(lc, lf, a[:1], a[1:], dt[:1], dt[1:])
+    torch.cuda.synchronize()
+    assert cp.status() == (0, 0) and fp.status() == (0, 0)
+    cn, fn, _, _ = oracle.amr_step(w.level, fine, P, cs, fs, cg, fg, a_old=a0, a_new=a1,
+                                   dt=dt[0].item())
+    assert _norm_rel(cp.from_device(lc.current, 6), cn) <= 1e-12
+    assert _norm_rel(fp.from_device(lf.current, 6), fn) <= 1e-12
+    amr.close(); fp.close(); cp.close()

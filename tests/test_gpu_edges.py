@@ -2,8 +2,9 @@
 down to single planes, ghost rectangles and flattening columns cut into
 pieces, scheme variants with their own instantiation, non-finite fluxes, and
 the mixed Poisson solve on grids that its tiles do not divide, with other
-sweep counts, from a given potential and at scales that fixed point cannot
-hold."""
+sweep counts, from a given potential, at scales that fixed point cannot hold,
+at tolerances near rounding, on a long domain, with a second solver alive and
+without memory for its fused form."""
 import itertools
 
 import numpy as np

@@ -107,8 +107,8 @@ def test_self_gravity_step_matches_the_oracle():
 
 
 def test_mixed_refinement_matches_the_oracle():
-    """Iterative refinement (FP64 residual and update, FP32 V-cycles) reaches
-    the same FP64 stopping test as the oracle's FP64 multigrid, in about as
+    """Iterative refinement (residual and update in fixed point, FP32 V-cycles)
+    reaches the same stopping test as the oracle's FP64 multigrid, in about as
     many cycles.  Two solutions whose residuals are both below tol max|f|
     differ by L^-1 of at most 2 tol max|f|; with tol = 1e-12 on this 64^3
     grid that is far below the 1e-9 gates on phi and g written here."""
