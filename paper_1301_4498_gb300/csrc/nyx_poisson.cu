@@ -467,8 +467,10 @@ __global__ void k_pg_shift_fix(long long *y, long long n, int b) {
 }
 
 // Residual r = f - L phi of the finest grid as float, the max norm of it
-// (out[0]) and the high word of the largest |phi| (out[1]; |phi| is at most
-// (out[1] + 1) 2^32 units).
+// (out[0]) and the high word of the largest |phi| where that is above `top`
+// (out[1]; |phi| is at most (max(top, out[1]) + 1) 2^32 units).  top is the last
+// measurement, so that few warps touch the second address: an atomic a warp took
+// 1 to 3 us.
 // h^2 r = f 2^-K + 6 phi - (neighbours) keeps f's K extra bits where the sum of
 // the others leaves room for them (|.| < 2^(62-K)), else they are below its
 // rounding to float; c = 1 / (h^2 s).
@@ -479,7 +481,7 @@ __global__ void k_pg_shift_fix(long long *y, long long n, int b) {
 constexpr int kRfX = 32, kRfY = 8;
 __global__ void __launch_bounds__(kRfX *kRfY)
     k_pg_resid_fix(const unsigned long long *phi, const long long *f, Dims d, float c, int K,
-                   int zc, float *r, unsigned long long *out) {
+                   int zc, unsigned top, float *r, unsigned long long *out) {
   struct Cells {
     unsigned long long v[2];
   };
@@ -517,8 +519,8 @@ __global__ void __launch_bounds__(kRfX *kRfY)
         const unsigned long long x = fine ? (v << K) + (unsigned long long)(F & ((1ll << K) - 1)) : v;
         q[u] = from_fix((long long)x) * (fine ? cK : c);
         loc = fmaxf(loc, fabsf(q[u]));
-        const int top = (int)(mid.v[u] >> 32);
-        pm = max(pm, (unsigned)(top ^ (top >> 31)));
+        const int hw = (int)(mid.v[u] >> 32);
+        pm = max(pm, (unsigned)(hw ^ (hw >> 31)));
       }
       *reinterpret_cast<float2 *>(r + zb + o) = make_float2(q[0], q[1]);
       lo = mid;
@@ -529,7 +531,7 @@ __global__ void __launch_bounds__(kRfX *kRfY)
   pm = __reduce_max_sync(0xffffffffu, pm);
   if (threadIdx.x == 0) {
     atomic_max_pos(out, (double)loc);
-    if (pm > *reinterpret_cast<volatile unsigned long long *>(out + 1))
+    if (pm > top && pm > *reinterpret_cast<volatile unsigned long long *>(out + 1))
       atomicMax(out + 1, (unsigned long long)pm);
   }
 }
@@ -1202,7 +1204,7 @@ int resid_max(nyx_poisson *S, double *out, double *pmax = nullptr) {
     G.z = (g.d.n[2] + zc - 1) / zc;
     k_pg_resid_fix<<<G, dim3(kRfX, kRfY), 0, S->P->stream>>>(
         (const unsigned long long *)S->d_fix, (const long long *)g.f, g.d,
-        (float)(g.ih2 / (double)S->fix_s), S->fix_k, zc, g32.f, S->d_max);
+        (float)(g.ih2 / (double)S->fix_s), S->fix_k, zc, S->fix_top, g32.f, S->d_max);
   } else if (S->L32.empty()) {
     const Grid3 G = grid3(g.d.n[0], g.d.n[1], g.d.n[2]);
     k_pg_resid_max<<<G.g, G.b, 0, S->P->stream>>>(g.phi, g.f, g.d, g.ih2, S->d_max);
@@ -1214,7 +1216,7 @@ int resid_max(nyx_poisson *S, double *out, double *pmax = nullptr) {
   }
   S->launches += 1;
   if (int rc = read_max(S, out, S->fixed || pmax ? &second : nullptr)) return rc;
-  if (S->fixed) S->fix_top = (unsigned)second;
+  if (S->fixed) S->fix_top = std::max(S->fix_top, (unsigned)second);
   if (pmax) std::memcpy(pmax, &second, sizeof(double));
   return NYX_OK;
 }
@@ -1257,6 +1259,7 @@ void refine_fixed(nyx_poisson *S, double res) {
   S->launches += 1;
   S->fix_s = (float)std::ldexp(s, b);
   S->fix_k -= b;
+  S->fix_top = (S->fix_top + 1) << b;  // (below 2^28: the bound is below 2^60)
 }
 
 // One cycle: a V-cycle on phi (FP64), or a refinement step (FP32 V-cycle on
